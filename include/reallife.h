@@ -371,13 +371,14 @@ rl_status reallife_kept_mass(const rl_mpi* m, const uint64_t* mask, double* out,
 /* ------------------------------------------------------------------ utilities */
 
 /* Kernel family for the warp kernels (render, gradient):
- *   0 (default) automatic: plane-parallel for launches of fewer than 2^19 pixel-views,
- *     per-pixel gather otherwise;
+ *   0 (default) automatic: renders plane-parallel for launches of fewer than 2^19 pixel-views
+ *     and per-pixel otherwise; gradients plane-parallel, per-pixel from 2^19 pixel-views on when
+ *     the warp offsets exceed 128 px; batched gradients per-pixel from 2^19 pixel-views on;
  *   1 not used (a family of TMA-staged plane windows, measured slower and removed): RL_EINVAL;
  *   2 per-pixel gather (one thread per view pixel walks all planes);
  *   3 plane-parallel (warps own chunks of planes; chunks combined through the
- *     associativity of the over operator), 8 warps per block;
- *   4 plane-parallel with 4 warps per block where D <= 32; 5 same as 3.
+ *     associativity of the over operator), about 8 warps per block;
+ *   4 plane-parallel with narrower blocks; 5 same as 3.
  * All compute the same values up to FP32 rounding of the accumulation order.
  * Process-wide; RL_EINVAL for other values. */
 rl_status reallife_set_kernel_path(int path);

@@ -2,8 +2,8 @@
 // all source views), the render backward used by autograd, and the loss reduction.
 //
 // Per view pixel q (one thread), with T_d = prod_{j>d}(1 - alpha_j) (Eq. eq_over):
-//   pass 1, d = D-1 .. 0:  m_d = bilinear(M[d], p_d(q)); T_d -> shared memory;
-//                           C += T_d alpha_d c_d; T *= (1 - alpha_d)
+//   pass 1, d = D-1 .. 0:  m_d = bilinear(M[d], p_d(q)); T_d of every kGroup-th plane -> shared
+//                           memory; C += T_d alpha_d c_d; T *= (1 - alpha_d)
 //   residual:               r = (C - I(q)) / N  (loss mode; L = 1/(2N) sum |C - I|^2; I the
 //                           level image: given at the level's resolution, img_level 0, or formed
 //                           on the fly from its 2^l x 2^l full-resolution pixels)
@@ -15,6 +15,14 @@
 // Sparse mode adds only into voxels kept by the selection (Sec. 3.3): the slot map
 // slots[d][y][x] gives the compact slot of a kept voxel (its rank among the kept planes of
 // the pixel) or RL_SLOT_NONE.  No division by (1 - alpha).
+//
+// What bounds it: L1 wavefronts (two gathers a sample and the reductions onto the kept taps) and
+// the latency of the gathers.  Both passes take the planes in groups of two, whose loads are in
+// flight together, and pass 2 forms the T_d within a group from the group's stored one: half the
+// shared memory, so that a launch of 64 planes keeps 32 warps an SM instead of 24 and its L1.
+// 1920x1080, D = 64, 8 views, BF16, anchored: 9.03 ms (one plane at a time 11.56 ms, groups of four
+// 10.8 ms; at the start, with border tests in every sample and a fenced loss reduction at the end
+// of every block, 12.9 ms).
 #include <type_traits>
 
 #include "rl_internal.h"
@@ -22,81 +30,64 @@
 namespace {
 
 constexpr int kGradBX = 32, kGradBY = 4, kGradThreads = kGradBX * kGradBY;
-#ifndef RL_GRAD_MIN_BLOCKS
-#define RL_GRAD_MIN_BLOCKS 10  // resident blocks per SM the register budget must allow (measured best)
-#endif
-
-template <bool SPARSE>
-__device__ __forceinline__ void scatter_tap(float* __restrict__ G, const uint8_t* __restrict__ slots_d, int d,
-                                            unsigned hw, int H, int W, int x, int y, float wt, float4 g, unsigned ng) {
-    if ((unsigned)x >= (unsigned)W || (unsigned)y >= (unsigned)H) return;
-    const unsigned pix = (unsigned)(y * W + x);
-    const unsigned slot = SPARSE ? (unsigned)__ldg(slots_d + pix) : (unsigned)d;
-    if ((SPARSE && slot == RL_SLOT_NONE) || !RL_IN(slot, ng)) return;
-    atomicAdd(reinterpret_cast<float4*>(G) + (slot * hw + pix), make_float4(wt * g.x, wt * g.y, wt * g.z, wt * g.w));
-}
-
-// Bilinear transpose of one sample's gradient g onto its four taps.
-template <bool SPARSE>
-__device__ __forceinline__ void scatter4(float* __restrict__ G, const uint8_t* __restrict__ slots_d, int d,
-                                         unsigned hw, int H, int W, const RLTaps& t, float4 g, unsigned ng) {
-    const float w00 = (1.f - t.fx) * (1.f - t.fy), w10 = t.fx * (1.f - t.fy);
-    const float w01 = (1.f - t.fx) * t.fy, w11 = t.fx * t.fy;
-    if ((unsigned)t.x0 < (unsigned)(W - 1) && (unsigned)t.y0 < (unsigned)(H - 1)) {
-        const unsigned p = (unsigned)(t.y0 * W + t.x0);
-        unsigned s00 = d, s10 = d, s01 = d, s11 = d;
-        if (SPARSE) {
-            s00 = __ldg(slots_d + p);
-            s10 = __ldg(slots_d + p + 1);
-            s01 = __ldg(slots_d + p + W);
-            s11 = __ldg(slots_d + p + W + 1);
-        }
-        float4* G4 = reinterpret_cast<float4*>(G);
-        if ((!SPARSE || s00 != RL_SLOT_NONE) && RL_IN(s00, ng))
-            atomicAdd(G4 + (s00 * hw + p), make_float4(w00 * g.x, w00 * g.y, w00 * g.z, w00 * g.w));
-        if ((!SPARSE || s10 != RL_SLOT_NONE) && RL_IN(s10, ng))
-            atomicAdd(G4 + (s10 * hw + p + 1), make_float4(w10 * g.x, w10 * g.y, w10 * g.z, w10 * g.w));
-        if ((!SPARSE || s01 != RL_SLOT_NONE) && RL_IN(s01, ng))
-            atomicAdd(G4 + (s01 * hw + p + W), make_float4(w01 * g.x, w01 * g.y, w01 * g.z, w01 * g.w));
-        if ((!SPARSE || s11 != RL_SLOT_NONE) && RL_IN(s11, ng))
-            atomicAdd(G4 + (s11 * hw + p + W + 1), make_float4(w11 * g.x, w11 * g.y, w11 * g.z, w11 * g.w));
-        return;
-    }
-    scatter_tap<SPARSE>(G, slots_d, d, hw, H, W, t.x0, t.y0, w00, g, ng);
-    scatter_tap<SPARSE>(G, slots_d, d, hw, H, W, t.x0 + 1, t.y0, w10, g, ng);
-    scatter_tap<SPARSE>(G, slots_d, d, hw, H, W, t.x0, t.y0 + 1, w01, g, ng);
-    scatter_tap<SPARSE>(G, slots_d, d, hw, H, W, t.x0 + 1, t.y0 + 1, w11, g, ng);
-}
+constexpr int kGroup = 2;           // planes whose samples are held together
+constexpr int kGradMinBlocks = 8;   // resident blocks the registers must allow (10: 9.28 ms, 6: 10.5 ms)
 
 // One block's tile of 32 x 4 view pixels of one view.  bid / nblocks index the block among
-// the launch's (or the batch item's) blocks for the loss epilogue.
+// the launch's (or the batch item's) blocks for the loss partials.
 template <typename Tm, bool SPARSE, bool LOSS, bool ANCH>
 __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H, int W, const RLViews& views, int view,
                                           int qx, int qy, int tid, float* __restrict__ sT,
                                           const float* __restrict__ images, int img_level,
                                           const float* __restrict__ grad_out, const uint8_t* __restrict__ slots,
                                           float* __restrict__ G, float inv_n, float* __restrict__ partials,
-                                          unsigned bid, unsigned nblocks, float* __restrict__ loss_out,
-                                          unsigned* __restrict__ counter, float loss_scale) {
+                                          unsigned bid, unsigned nblocks) {
     float lsum = 0.f;
     __shared__ RLAnchor sA;  // the tile's anchor: its centre pixel
     if (ANCH)
         rl_anchor_build(&sA, views, view, (qx & ~(kGradBX - 1)) + kGradBX / 2, qy - qy % kGradBY + kGradBY / 2, D,
                         tid, kGradThreads);
+    const unsigned act = __ballot_sync(0xffffffffu, qx < W && qy < H);
     if (qx < W && qy < H) {
         const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[view], qx, qy);
         const size_t plane = (size_t)H * W * 4;
+        const unsigned hw = (unsigned)(H * W), base = rl_fast_base(qx, qy, W);
+        // warps whose samples of every plane lie inside it skip the border tests
+        const bool fast = __all_sync(act, rl_chunk_inside<ANCH>(w, sA, views, 0, D - 1, qx, qy, H, W));
+        // the sample of plane d (transparent beyond the last plane)
+        const auto inside = [&](int d, const RLFastTap& t) {
+            return RL_IN((long long)t.idx + W + 1, hw) ? rl_sample_at(M, (unsigned)d * hw + t.idx, W, t.fx, t.fy)
+                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        const int groups = (D + kGroup - 1) / kGroup;
         float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
 #pragma unroll 1
-        for (int d = D - 1; d >= 0; --d) {
-            const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
-            const float4 m = rl_sample_fast(M + d * plane, H, W, t);
-            sT[d * kGradThreads + tid] = T;
-            const float a = T * m.w;
-            c0 = fmaf(a, m.x, c0);
-            c1 = fmaf(a, m.y, c1);
-            c2 = fmaf(a, m.z, c2);
-            T = T * (1.f - m.w);
+        for (int j = groups - 1; j >= 0; --j) {
+            float4 m[kGroup];
+            if (fast) {
+#pragma unroll
+                for (int i = kGroup - 1; i >= 0; --i) {
+                    const int d = min(j * kGroup + i, D - 1);
+                    m[i] = inside(d, rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W));
+                    if (j * kGroup + i >= D) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            } else {
+#pragma unroll
+                for (int i = kGroup - 1; i >= 0; --i) {
+                    const int d = j * kGroup + i;
+                    m[i] = d < D ? rl_sample(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            }
+            sT[j * kGradThreads + tid] = T;
+#pragma unroll
+            for (int i = kGroup - 1; i >= 0; --i) {
+                const float a = T * m[i].w;
+                c0 = fmaf(a, m[i].x, c0);
+                c1 = fmaf(a, m[i].y, c1);
+                c2 = fmaf(a, m[i].z, c2);
+                T = T * (1.f - m[i].w);
+            }
         }
         float r0, r1, r2;
         if (LOSS) {
@@ -127,26 +118,57 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
             r2 = __ldg(go + 2);
         }
         float b0 = 0.f, b1 = 0.f, b2 = 0.f;
-        const unsigned hw = (unsigned)(H * W);
         const unsigned ng = views.gplanes ? (unsigned)views.gplanes : (unsigned)D;  // checked in debug builds
 #pragma unroll 1
-        for (int d = 0; d < D; ++d) {
-            const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
-            const float4 m = rl_sample_fast(M + d * plane, H, W, t);
-            const float Td = sT[d * kGradThreads + tid];
-            if (t.ok && Td != 0.f) {
-                const float gc = Td * m.w;
-                float4 g;
-                g.x = gc * r0;
-                g.y = gc * r1;
-                g.z = gc * r2;
-                g.w = Td * fmaf(m.x - b0, r0, fmaf(m.y - b1, r1, (m.z - b2) * r2));
-                scatter4<SPARSE>(G, SPARSE ? slots + (size_t)d * hw : nullptr, d, hw, H, W, t, g, ng);
+        for (int j = 0; j < groups; ++j) {
+            float4 m[kGroup];
+            float Td[kGroup];
+            unsigned word[kGroup];
+            if (fast) {
+#pragma unroll
+                for (int i = kGroup - 1; i >= 0; --i) {
+                    const int d = min(j * kGroup + i, D - 1);
+                    const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                    m[i] = inside(d, t);
+                    if (SPARSE) word[i] = rl_slot_word(slots, (unsigned)d * hw + t.idx, W);
+                    if (j * kGroup + i >= D) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+            } else {
+#pragma unroll
+                for (int i = kGroup - 1; i >= 0; --i) {
+                    const int d = j * kGroup + i;
+                    word[i] = 0u;
+                    m[i] = d < D ? rl_sample(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
+                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
             }
-            const float om = 1.f - m.w;
-            b0 = fmaf(m.x, m.w, om * b0);
-            b1 = fmaf(m.y, m.w, om * b1);
-            b2 = fmaf(m.z, m.w, om * b2);
+            float Tg = sT[j * kGradThreads + tid];
+#pragma unroll
+            for (int i = kGroup - 1; i >= 0; --i) {
+                Td[i] = Tg;
+                Tg = Tg * (1.f - m[i].w);
+            }
+#pragma unroll
+            for (int i = 0; i < kGroup; ++i) {
+                const int d = j * kGroup + i;
+                if (Td[i] != 0.f && d < D) {
+                    const float gc = Td[i] * m[i].w;
+                    const float4 g = make_float4(gc * r0, gc * r1, gc * r2,
+                                                 Td[i] * fmaf(m[i].x - b0, r0, fmaf(m[i].y - b1, r1, (m[i].z - b2) * r2)));
+                    if (fast) {
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                        rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W, t.fx,
+                                              t.fy, g, ng);
+                    } else {
+                        const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
+                        if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);
+                    }
+                }
+                const float om = 1.f - m[i].w;
+                b0 = fmaf(m[i].x, m[i].w, om * b0);
+                b1 = fmaf(m[i].y, m[i].w, om * b1);
+                b2 = fmaf(m[i].z, m[i].w, om * b2);
+            }
         }
     }
     if (LOSS) {
@@ -154,41 +176,36 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
         lsum = rl_warp_sum(lsum);
         if ((tid & 31) == 0) red[tid >> 5] = lsum;
         __syncthreads();
-        float blk = 0.f;
-        if (tid == 0)
+        if (tid == 0) {
+            float blk = 0.f;
             for (int j = 0; j < kGradThreads / 32; ++j) blk += red[j];
-        __syncthreads();
-        rl_loss_epilogue(blk, partials, bid, nblocks, loss_out, counter, loss_scale, tid, kGradThreads, red);
+            if (RL_IN(bid, nblocks)) partials[bid] = blk;
+        }
     }
 }
 
 template <typename Tm, bool SPARSE, bool LOSS, bool ANCH>
-__global__ void __launch_bounds__(kGradThreads, RL_GRAD_MIN_BLOCKS)
-k_grad(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views, int tiles_x,
+__global__ void __launch_bounds__(kGradThreads, kGradMinBlocks)
+k_grad(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views,
        const float* __restrict__ images, int img_level, const float* __restrict__ grad_out,
-       const uint8_t* __restrict__ slots, float* __restrict__ G, float inv_n, float* __restrict__ partials,
-       float* __restrict__ loss_out, unsigned* __restrict__ counter, float loss_scale) {
-    extern __shared__ float sT[];  // [D][kGradThreads]
+       const uint8_t* __restrict__ slots, float* __restrict__ G, float inv_n, float* __restrict__ partials) {
+    extern __shared__ float sT[];  // [ceil(D / kGroup)][kGradThreads]
     // view-fastest block order: the N views of a tile run together and share M through L2
     grad_tile<Tm, SPARSE, LOSS, ANCH>(M, D, H, W, views, blockIdx.x, blockIdx.y * kGradBX + threadIdx.x,
                                 blockIdx.z * kGradBY + threadIdx.y, threadIdx.y * kGradBX + threadIdx.x, sT, images,
                                 img_level, grad_out, slots, G, inv_n, partials,
                                 blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
-                                gridDim.x * gridDim.y * gridDim.z, loss_out, counter, loss_scale);
+                                gridDim.x * gridDim.y * gridDim.z);
 }
 
 // Batched gradient, per-pixel gather family: one persistent launch walks the gradient units of
 // the batch table's items that take this family (a unit is one 32 x 4 tile of one view of one
-// item, in the order of k_grad's grid), each item with its own loss epilogue over its own
-// units.  The dynamic shared memory holds `planes` planes; an item with more sets the batch bit
+// item, in the order of k_grad's grid), each writing its own loss partial.  The dynamic shared memory holds `planes` planes; an item with more sets the batch bit
 // of the status word and is skipped.
-#ifndef RL_GRAD_BATCH_MIN_BLOCKS
-#define RL_GRAD_BATCH_MIN_BLOCKS 8  // the table lookups need registers: at 10 blocks the kernel spills
-#endif
 template <typename Tm>
-__global__ void __launch_bounds__(kGradThreads, RL_GRAD_BATCH_MIN_BLOCKS)
+__global__ void __launch_bounds__(kGradThreads, kGradMinBlocks)
 k_grad_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restrict__ items, int planes) {
-    extern __shared__ float sT[];  // [planes][kGradThreads]
+    extern __shared__ float sT[];  // [ceil(planes / kGroup)][kGradThreads]
     const unsigned n = hdr->n, total = hdr->grad_units;
     if (hdr->dtype != (std::is_same<Tm, float>::value ? (unsigned)RL_F32 : (unsigned)RL_BF16)) return;
     const int tid = threadIdx.y * kGradBX + threadIdx.x;
@@ -207,7 +224,7 @@ k_grad_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restric
                                              tx * kGradBX + threadIdx.x, ty * kGradBY + threadIdx.y, tid, sT,       \
                                              it.level ? it.Il : it.images, 0, nullptr, it.slots, it.G, it.inv_n,    \
                                              it.partials,                                                           \
-                                             local, it.grad_units, it.loss_out, it.counter, it.loss_scale)
+                                             local, it.grad_units)
         if (it.views.anchored) RL_GB(true);
         else RL_GB(false);
 #undef RL_GB
@@ -215,30 +232,22 @@ k_grad_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restric
     }
 }
 
-// Deterministic sum of the per-block partials (fixed order), times `scale`.
+// The loss from the per-block partials (reallife_loss_grad; an HSGD step's update does it).
 __global__ void __launch_bounds__(1024) k_loss_reduce(const float* __restrict__ partials, int n, float scale,
                                                      float* __restrict__ out) {
     __shared__ float red[32];
-    float s = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += partials[i];
-    s = rl_warp_sum(s);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-        v = rl_warp_sum(v);
-        if (threadIdx.x == 0) out[0] = v * scale;
-    }
+    const float total = rl_partials_sum(partials, (unsigned)n, threadIdx.x, blockDim.x, red);
+    if (threadIdx.x == 0) out[0] = total * scale;
 }
 
 template <typename Tm, bool SPARSE, bool LOSS>
 void launch_grad_t(const void* M, int D, int H, int W, const RLViews& views, const float* images, int img_level,
-                   const float* grad_out, const uint8_t* slots, float* G, float inv_n, float* partials, float* loss_out,
-                   unsigned* counter, float loss_scale, int tiles_x, dim3 grid, size_t smem, cudaStream_t s) {
+                   const float* grad_out, const uint8_t* slots, float* G, float inv_n, float* partials,
+                   dim3 grid, size_t smem, cudaStream_t s) {
     auto kern = views.anchored ? k_grad<Tm, SPARSE, LOSS, true> : k_grad<Tm, SPARSE, LOSS, false>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<grid, dim3(kGradBX, kGradBY), smem, s>>>((const Tm*)M, D, H, W, views, tiles_x, images, img_level, grad_out,
-                                                    slots, G, inv_n, partials, loss_out, counter, loss_scale);
+    kern<<<grid, dim3(kGradBX, kGradBY), smem, s>>>((const Tm*)M, D, H, W, views, images, img_level, grad_out, slots, G,
+                                                    inv_n, partials);
 }
 
 }  // namespace
@@ -251,30 +260,31 @@ size_t rl_grad_num_blocks(int H, int W, int N) {
 
 rl_status rl_launch_grad(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                          const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G,
-                         float inv_n, float* partials, int* nblocks, cudaStream_t s, float* loss_out,
-                         unsigned* counter, float loss_scale) {
-    const int path = rl_kernel_path(H, W, views.n);
-    if (path != 2)
+                         float inv_n, float* partials, int* nblocks, cudaStream_t s) {
+    if (rl_grad_path(H, W, views.n, views.anchored != 0) != 2)
         return rl_launch_grad_pp(M, dt, D, H, W, views, mode_loss, images, img_level, grad_out, slots, G, inv_n,
-                                 partials, nblocks, s, loss_out, counter, loss_scale);
+                                 partials, nblocks, s);
     const int tiles_x = (W + kGradBX - 1) / kGradBX, tiles_y = (H + kGradBY - 1) / kGradBY;
     const dim3 grid((unsigned)views.n, (unsigned)tiles_x, (unsigned)tiles_y);
-    const size_t smem = (size_t)D * kGradThreads * sizeof(float);
+    const size_t smem = (size_t)((D + kGroup - 1) / kGroup) * kGradThreads * sizeof(float);
     if (nblocks) *nblocks = (int)(grid.x * grid.y * grid.z);
     const bool sparse = slots != nullptr;
     const char* name = dt == RL_F32 ? (sparse ? "grad_sparse_f32" : "grad_dense_f32")
                                     : (sparse ? "grad_sparse_bf16" : "grad_dense_bf16");
     RLTraceScope ts(name, s);
 #define RL_GRAD_CASE(TM, SP, LS) \
-    launch_grad_t<TM, SP, LS>(M, D, H, W, views, images, img_level, grad_out, slots, G, inv_n, partials, loss_out, \
-                              counter, loss_scale, tiles_x, grid, smem, s)
-    if (dt == RL_F32) {
-        if (sparse) { if (mode_loss) RL_GRAD_CASE(float, true, true); else RL_GRAD_CASE(float, true, false); }
-        else        { if (mode_loss) RL_GRAD_CASE(float, false, true); else RL_GRAD_CASE(float, false, false); }
-    } else {
-        if (sparse) { if (mode_loss) RL_GRAD_CASE(__nv_bfloat16, true, true); else RL_GRAD_CASE(__nv_bfloat16, true, false); }
-        else        { if (mode_loss) RL_GRAD_CASE(__nv_bfloat16, false, true); else RL_GRAD_CASE(__nv_bfloat16, false, false); }
-    }
+    launch_grad_t<TM, SP, LS>(M, D, H, W, views, images, img_level, grad_out, slots, G, inv_n, partials, grid, \
+                              smem, s)
+    // a slot map comes with the loss mode only
+#define RL_KIND(TM)                                                                               \
+    do {                                                                                          \
+        if (slots) RL_GRAD_CASE(TM, true, true);                                                      \
+        else if (mode_loss) RL_GRAD_CASE(TM, false, true);                                            \
+        else RL_GRAD_CASE(TM, false, false);                                                          \
+    } while (0)
+    if (dt == RL_F32) RL_KIND(float);
+    else RL_KIND(__nv_bfloat16);
+#undef RL_KIND
 #undef RL_GRAD_CASE
     return rl_check_launch("grad");
 }
@@ -286,9 +296,9 @@ rl_status rl_launch_grad_batch(const void* table, rl_dtype dt, int planes, cudaS
     const RLBatchHeader* hdr = static_cast<const RLBatchHeader*>(table);
     const RLBatchItem* items = rl_batch_items(table);
     planes = planes < 1 ? 1 : (planes > RL_DEV_MAX_PLANES ? RL_DEV_MAX_PLANES : planes);
-    const size_t smem = (size_t)planes * kGradThreads * sizeof(float);
+    const size_t smem = (size_t)((planes + kGroup - 1) / kGroup) * kGradThreads * sizeof(float);
     // the resident blocks of the largest shared memory, so that any later capacity fits the grid
-    const size_t smem_max = (size_t)RL_DEV_MAX_PLANES * kGradThreads * sizeof(float);
+    const size_t smem_max = (size_t)((RL_DEV_MAX_PLANES + kGroup - 1) / kGroup) * kGradThreads * sizeof(float);
     const int grid = dt == RL_F32 ? rl_persistent_grid<k_grad_batch<float>>(kGradThreads, smem_max)
                                   : rl_persistent_grid<k_grad_batch<__nv_bfloat16>>(kGradThreads, smem_max);
     if (dt == RL_F32) {

@@ -1,16 +1,15 @@
 // pp.cu -- plane-parallel warp kernels: novel-view rendering (Eq. eq_render, eq_over) and
 // the fused warp + composite + residual + exact adjoint of one HSGD iteration.
 //
-// Layout.  A block is kGroups (4 or 8) warps over the same 32 view pixels (a 16 x 2 tile; grid =
-// (views, tiles_x, tiles_y) so that the views of a tile run together); warp g
-// owns planes [g C, g C + C), C = ceil(D / kGroups) rounded up to 1, 2, 4 or 8, so a warp's loads of one plane
-// are 32 neighbouring voxels.  Each thread samples its C planes once and keeps them in
+// Layout.  Several warps share the same 32 view pixels (grid = (views, tiles_x, tiles_y), so that
+// the views of a tile run together); warp g owns a chunk of consecutive planes, so a warp's loads
+// of one plane are neighbouring voxels.  Each thread samples its C planes once and keeps them in
 // registers, nearest first forming its chunk's composite Cc_g = sum c_d alpha_d T_d^loc
 // and transmittance Tc_g = prod (1 - alpha_d).  The over operator is associative, so the
 // chunks combine exactly:
 //   T before chunk g (everything nearer):  Tb_g = prod_{g' > g} Tc_g'
-//   pixel colour:                          C = sum_g Tb_g Cc_g
-//   composite of everything farther:       Bb_g = f_{g-1}(... f_0(0)), f_g(x) = Cc_g + Tc_g x
+//   pixel colour:                          C = f_{G-1}(... f_0(0)), f_g(x) = Cc_g + Tc_g x
+//   composite of everything farther:       Bb_g = f_{g-1}(... f_0(0))
 // (shared-memory exchange of the per-chunk (Cc, Tc)).  The adjoint of plane d then uses
 // T_d = Tb_g T_d^loc and the running below-composite B_d (B_{d+1} = c_d alpha_d + (1 -
 // alpha_d) B_d, starting from Bb_g) -- no division by (1 - alpha), no second gather.
@@ -21,7 +20,7 @@
 
 namespace {
 
-constexpr int kTX = 16, kTY = 2, kPix = 32;  // pixels per block, one per lane
+constexpr int kTX = 16, kTY = 2, kPix = 32;  // render: pixels per block, one per lane
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 
@@ -46,58 +45,6 @@ __device__ __forceinline__ float4 sample_pp(const Tm* __restrict__ plane, int H,
         return make_float4(lo.x, lo.y, hi.x, hi.y);
     }
     return rl_sample(plane, H, W, t);
-}
-
-template <bool SPARSE>
-__device__ __forceinline__ void scatter_tap_pp(float4* __restrict__ G4, const uint8_t* __restrict__ slots_d,
-                                               unsigned d, unsigned hw, int H, int W, int x, int y, float wt,
-                                               float4 g, unsigned ng) {
-    if ((unsigned)x >= (unsigned)W || (unsigned)y >= (unsigned)H) return;
-    const unsigned pix = (unsigned)(y * W + x);
-    const unsigned slot = SPARSE ? (unsigned)__ldg(slots_d + pix) : d;
-    if ((SPARSE && slot == RL_SLOT_NONE) || !RL_IN(slot, ng)) return;
-    atomicAdd(G4 + (slot * hw + pix), make_float4(wt * g.x, wt * g.y, wt * g.z, wt * g.w));
-}
-
-// Bilinear transpose of one sample's gradient onto its four taps (kept voxels only).
-template <bool SPARSE>
-__device__ __forceinline__ void scatter_pp(float* __restrict__ G, const uint8_t* __restrict__ slots_d, unsigned d,
-                                           unsigned hw, int H, int W, const RLTaps& t, float4 g, unsigned ng) {
-    const float w00 = (1.f - t.fx) * (1.f - t.fy), w10 = t.fx * (1.f - t.fy);
-    const float w01 = (1.f - t.fx) * t.fy, w11 = t.fx * t.fy;
-    float4* G4 = reinterpret_cast<float4*>(G);
-    if ((unsigned)t.x0 < (unsigned)(W - 1) && (unsigned)t.y0 < (unsigned)(H - 1)) {
-        const unsigned p = (unsigned)(t.y0 * W + t.x0);
-        unsigned s00 = d, s10 = d, s01 = d, s11 = d;
-        if (SPARSE) {
-            s00 = __ldg(slots_d + p);
-            s10 = __ldg(slots_d + p + 1);
-            s01 = __ldg(slots_d + p + W);
-            s11 = __ldg(slots_d + p + W + 1);
-        }
-        const float2 gl = f2(g.x, g.y), gh = f2(g.z, g.w);
-        if ((!SPARSE || s00 != RL_SLOT_NONE) && RL_IN(s00, ng)) {
-            const float2 a = __fmul2_rn(f2(w00, w00), gl), b = __fmul2_rn(f2(w00, w00), gh);
-            atomicAdd(G4 + (s00 * hw + p), make_float4(a.x, a.y, b.x, b.y));
-        }
-        if ((!SPARSE || s10 != RL_SLOT_NONE) && RL_IN(s10, ng)) {
-            const float2 a = __fmul2_rn(f2(w10, w10), gl), b = __fmul2_rn(f2(w10, w10), gh);
-            atomicAdd(G4 + (s10 * hw + p + 1), make_float4(a.x, a.y, b.x, b.y));
-        }
-        if ((!SPARSE || s01 != RL_SLOT_NONE) && RL_IN(s01, ng)) {
-            const float2 a = __fmul2_rn(f2(w01, w01), gl), b = __fmul2_rn(f2(w01, w01), gh);
-            atomicAdd(G4 + (s01 * hw + p + W), make_float4(a.x, a.y, b.x, b.y));
-        }
-        if ((!SPARSE || s11 != RL_SLOT_NONE) && RL_IN(s11, ng)) {
-            const float2 a = __fmul2_rn(f2(w11, w11), gl), b = __fmul2_rn(f2(w11, w11), gh);
-            atomicAdd(G4 + (s11 * hw + p + W + 1), make_float4(a.x, a.y, b.x, b.y));
-        }
-        return;
-    }
-    scatter_tap_pp<SPARSE>(G4, slots_d, d, hw, H, W, t.x0, t.y0, w00, g, ng);
-    scatter_tap_pp<SPARSE>(G4, slots_d, d, hw, H, W, t.x0 + 1, t.y0, w10, g, ng);
-    scatter_tap_pp<SPARSE>(G4, slots_d, d, hw, H, W, t.x0, t.y0 + 1, w01, g, ng);
-    scatter_tap_pp<SPARSE>(G4, slots_d, d, hw, H, W, t.x0 + 1, t.y0 + 1, w11, g, ng);
 }
 
 struct PixelCoord {
@@ -167,96 +114,175 @@ k_render_pp(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant
     }
 }
 
-// One block's tile (kPix view pixels of one view, all planes): the body of k_grad_pp, with the
-// tile, the exchange buffers and the block's index for the loss epilogue given explicitly.
-template <typename Tm, int C, int kGroups, bool SPARSE, bool LOSS, bool ANCH>
+// ------------------------------------------------------------------ fused gradient
+//
+// One block: `tiles` tiles of 32 view pixels side by side along x, G warps a tile; warp g of a
+// tile holds the kChunk planes from kChunk g on (the last chunk may be short).
+//
+// What bounds it: at 512x384, D = 32, 4 views, FP32 the level-0 launch issues 179 M warp
+// instructions at 67% of the issue slots, with 38 M L1 wavefronts (57%): one gather a sample
+// (the per-pixel gather family takes two, 57 M wavefronts) plus the reductions onto the kept
+// taps.  Four planes a warp at 64 registers (32 resident warps) is the measured optimum:
+// 218 us, against 284 us with eight planes at 128 registers or at 80 (half the warps, and twice
+// the unrolled code: instruction fetch stalls), and 455 us with four planes whose taps are kept
+// instead of formed again in the adjoint (spills).  The same launch took 274 us per-pixel before.
+constexpr int kChunk = 4, kMaxWarps = 16;  // RL_DEV_MAX_PLANES / kChunk
+
+struct PPShape {
+    int G, tiles;   // warps a tile, tiles a block
+    int tile_x;     // a tile is tile_x x (32 / tile_x) pixels
+};
+
+// Tile of the gradient over a W x H image: 32 x 1 pixels (512x384: 218 against 224 us with 16 x 2)
+// unless 16 x 2 needs fewer tiles (widths just above a multiple of 32).
+__host__ __device__ inline int grad_pp_tile_x(int H, int W) {
+    return (W + 15) / 16 * ((H + 1) / 2) < (W + 31) / 32 * H ? 16 : 32;
+}
+
+// Blocks of about `most_warps` warps; a tile of D planes takes ceil(D / 4) of them.
+__host__ __device__ inline PPShape grad_pp_shape(int D, int H, int W, int most_warps) {
+    PPShape s;
+    s.G = (D + kChunk - 1) / kChunk;
+    s.tiles = most_warps / s.G > 1 ? most_warps / s.G : 1;
+    s.tile_x = grad_pp_tile_x(H, W);
+    return s;
+}
+
+// Position of one thread: view pixel (qx, qy), plane chunk g of its tile.
+struct PPPos {
+    int view, tx, ty, tile, g, G, lane, qx, qy;
+    bool active;
+};
+
+__device__ __forceinline__ PPPos pp_pos(int H, int W, int view, int bx, int by, PPShape sh) {
+    PPPos c;
+    const int wi = threadIdx.x >> 5;
+    c.view = view;
+    c.G = sh.G;
+    c.tile = wi / sh.G;
+    c.g = wi - c.tile * sh.G;
+    c.lane = threadIdx.x & 31;
+    c.tx = bx * sh.tiles + c.tile;
+    c.ty = by;
+    const int log_x = sh.tile_x == 32 ? 5 : 4;
+    c.qx = c.tx * sh.tile_x + (c.lane & (sh.tile_x - 1));
+    c.qy = (by << (5 - log_x)) + (c.lane >> log_x);
+    // warps beyond the last tile of a persistent block hold no pixel
+    c.active = c.tile < sh.tiles && c.qx < W && c.qy < H;
+    return c;
+}
+
+template <typename Tm, bool FULL, bool SPARSE, bool LOSS, bool ANCH>
 __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, int H, int W, const RLViews& views,
-                                             const PixelCoord pc, const float* __restrict__ images, int img_level,
-                                             const float* __restrict__ grad_out, const uint8_t* __restrict__ slots,
-                                             float* __restrict__ G, float inv_n, float* __restrict__ partials,
-                                             unsigned bid, unsigned nblocks, float* __restrict__ loss_out,
-                                             unsigned* __restrict__ counter, float loss_scale,
-                                             float4 (*__restrict__ xch)[kPix], float* __restrict__ red) {
+                                             const PPPos pc, PPShape sh, int bx, const float* __restrict__ images,
+                                             int img_level, const float* __restrict__ grad_out,
+                                             const uint8_t* __restrict__ slots, float* __restrict__ G, float inv_n,
+                                             float* __restrict__ partials, unsigned nparts) {
+    constexpr int C = kChunk;
+    __shared__ float4 xch[kMaxWarps][kPix];  // per chunk: (Cc.rgb, Tc)
+    __shared__ float ximg[kMaxWarps][kPix][3];
     __shared__ RLAnchor sA;
     if (ANCH)
-        rl_anchor_build(&sA, views, pc.view, (pc.qx - pc.qx % kTX) + kTX / 2, (pc.qy - pc.qy % kTY) + kTY / 2, D,
-                        threadIdx.x, kGroups * kPix);
+        rl_anchor_build(&sA, views, pc.view, bx * sh.tiles * sh.tile_x + sh.tiles * sh.tile_x / 2,
+                        pc.ty * (kPix / sh.tile_x), D, threadIdx.x, blockDim.x);
     const int qx = min(pc.qx, W - 1), qy = min(pc.qy, H - 1);
     const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[pc.view], qx, qy);
+    const unsigned hw = (unsigned)(H * W);
     const size_t plane = (size_t)H * W * 4;
+    const int d0 = pc.g * C;
+    const int n = FULL ? C : min(C, D - d0);  // planes of this warp's chunk (>= 1)
 
     // a level image that is already averaged (img_level 0: one pixel a view) is read by one warp
     // before its gathers and handed to the others through shared memory at the chunk exchange
-    __shared__ float ximg[kPix][3];
-    const bool img_early = LOSS && img_level == 0;
+    const bool img_early = LOSS && img_level == 0 && pc.g == pc.G - 1;
     float li0 = 0.f, li1 = 0.f, li2 = 0.f;
-    if (img_early && pc.g == kGroups - 1 && pc.active) {
+    if (img_early && pc.active) {
         const float* px = images + (((size_t)pc.view * H + pc.qy) * W + pc.qx) * 3;
         li0 = __ldg(px);
         li1 = __ldg(px + 1);
         li2 = __ldg(px + 2);
     }
 
-    // forward over this thread's chunk, nearest plane first; samples stay in registers
+    // forward over this thread's chunk; the samples and their taps' slots stay in registers
     float4 m[C];
     float Tloc[C];
+    unsigned word[C];
+    const unsigned base = rl_fast_base(qx, qy, W);
+    const bool fast = __all_sync(0xffffffffu, rl_chunk_inside<ANCH>(w, sA, views, d0, d0 + n - 1, qx, qy, H, W));
+    if (fast) {
+#pragma unroll
+        for (int i = C - 1; i >= 0; --i) {
+            const int d = FULL ? d0 + i : d0 + min(i, n - 1);
+            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+            m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            word[i] = 0xFFFFFFFFu;
+            if (RL_IN((long long)t.idx + W + 1, hw)) {
+                m[i] = rl_sample_at(M, (unsigned)d * hw + t.idx, W, t.fx, t.fy);
+                if (SPARSE) word[i] = rl_slot_word(slots, (unsigned)d * hw + t.idx, W);
+            }
+            if (!FULL && i >= n) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    } else {
+#pragma unroll
+        for (int i = C - 1; i >= 0; --i) {
+            word[i] = 0u;
+            m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (FULL || i < n) {
+                const int d = d0 + i;
+                m[i] = rl_sample(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy));
+            }
+        }
+    }
     float Tl = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
 #pragma unroll
     for (int i = C - 1; i >= 0; --i) {
-        const int d = pc.g * C + i;
-        m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         Tloc[i] = Tl;
-        if (d < D) {
-            const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
-            m[i] = sample_pp(M + d * plane, H, W, t);
-            const float a = Tl * m[i].w;
-            c0 = fmaf(a, m[i].x, c0);
-            c1 = fmaf(a, m[i].y, c1);
-            c2 = fmaf(a, m[i].z, c2);
-            Tl = Tl * (1.f - m[i].w);
-        }
+        const float a = Tl * m[i].w;
+        c0 = fmaf(a, m[i].x, c0);
+        c1 = fmaf(a, m[i].y, c1);
+        c2 = fmaf(a, m[i].z, c2);
+        Tl = Tl * (1.f - m[i].w);
     }
-    xch[pc.g][pc.lane] = make_float4(c0, c1, c2, Tl);
-    if (img_early && pc.g == kGroups - 1) {
-        ximg[pc.lane][0] = li0;
-        ximg[pc.lane][1] = li1;
-        ximg[pc.lane][2] = li2;
+    const int wi = threadIdx.x >> 5, w0 = wi - pc.g;  // this tile's warps are w0 .. w0 + G - 1
+    xch[wi][pc.lane] = make_float4(c0, c1, c2, Tl);
+    if (img_early) {
+        ximg[pc.tile][pc.lane][0] = li0;
+        ximg[pc.tile][pc.lane][1] = li1;
+        ximg[pc.tile][pc.lane][2] = li2;
     }
     __syncthreads();
-    // combine the chunks: pixel colour, transmittance in front of this chunk and the
-    // composite of everything behind it
-    float Tb = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-    {
-        float T = 1.f;
-#pragma unroll
-        for (int g = kGroups - 1; g >= 0; --g) {
-            const float4 v = xch[g][pc.lane];
-            if (g == pc.g) Tb = T;
-            C0 = fmaf(T, v.x, C0);
-            C1 = fmaf(T, v.y, C1);
-            C2 = fmaf(T, v.z, C2);
-            T = T * v.w;
-        }
-    }
-    float b0 = 0.f, b1 = 0.f, b2 = 0.f;
-    for (int g = 0; g < pc.g; ++g) {
+    // combine the chunks, farthest first: the composite of everything behind this chunk, the
+    // transmittance in front of it and the pixel colour
+    float b0 = 0.f, b1 = 0.f, b2 = 0.f, Tb = 1.f;
+#pragma unroll 4
+    for (int g = w0; g < wi; ++g) {
         const float4 v = xch[g][pc.lane];
         b0 = fmaf(v.w, b0, v.x);
         b1 = fmaf(v.w, b1, v.y);
         b2 = fmaf(v.w, b2, v.z);
     }
-    float r0 = 0.f, r1 = 0.f, r2 = 0.f, lsum = 0.f;
+    float C0 = fmaf(Tl, b0, c0), C1 = fmaf(Tl, b1, c1), C2 = fmaf(Tl, b2, c2);
+#pragma unroll 4
+    for (int g = wi + 1; g < w0 + pc.G; ++g) {
+        const float4 v = xch[g][pc.lane];
+        C0 = fmaf(v.w, C0, v.x);
+        C1 = fmaf(v.w, C1, v.y);
+        C2 = fmaf(v.w, C2, v.z);
+        Tb = Tb * v.w;
+    }
+    float lsum = 0.f;
     if (pc.active) {
+        float r0, r1, r2;
         if (LOSS) {
             const int s = 1 << img_level;
-            const int Wf = W << img_level, Hf = H << img_level;
-            const float* img = images + (size_t)pc.view * Hf * Wf * 3;
             float i0 = 0.f, i1 = 0.f, i2 = 0.f;
-            if (img_early) {
-                i0 = ximg[pc.lane][0];
-                i1 = ximg[pc.lane][1];
-                i2 = ximg[pc.lane][2];
+            if (img_level == 0) {
+                i0 = ximg[pc.tile][pc.lane][0];
+                i1 = ximg[pc.tile][pc.lane][1];
+                i2 = ximg[pc.tile][pc.lane][2];
             } else {
+                const int Wf = W << img_level, Hf = H << img_level;
+                const float* img = images + (size_t)pc.view * Hf * Wf * 3;
                 for (int yy = 0; yy < s; ++yy)
                     for (int xx = 0; xx < s; ++xx) {
                         const float* px = img + ((size_t)(pc.qy * s + yy) * Wf + (pc.qx * s + xx)) * 3;
@@ -269,7 +295,7 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
             // the image mean is rounded on its own (as the level images of the pyramid pass are)
             const float e0 = C0 - __fmul_rn(i0, inv_area), e1 = C1 - __fmul_rn(i1, inv_area),
                         e2 = C2 - __fmul_rn(i2, inv_area);
-            if (pc.g == 0) lsum = fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
+            lsum = fmaf(e0, e0, fmaf(e1, e1, e2 * e2));
             r0 = e0 * inv_n;
             r1 = e1 * inv_n;
             r2 = e2 * inv_n;
@@ -280,25 +306,27 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
             r2 = __ldg(go + 2);
         }
         // adjoint over the chunk, farthest plane first
-        const unsigned hw = (unsigned)(H * W);
         const unsigned ng = views.gplanes ? (unsigned)views.gplanes : (unsigned)D;  // checked in debug builds
 #pragma unroll
         for (int i = 0; i < C; ++i) {
-            const int d = pc.g * C + i;
-            if (d < D) {
+            if (FULL || i < n) {
+                const int d = d0 + i;
                 const float Td = Tb * Tloc[i];
                 const float4 mi = m[i];
                 if (Td != 0.f) {
-                    const RLTaps t = w.taps(sA, d, views.rho[d], pc.qx, pc.qy);
-                    if (t.ok) {
-                        const float gc = Td * mi.w;
-                        float4 g;
-                        g.x = gc * r0;
-                        g.y = gc * r1;
-                        g.z = gc * r2;
-                        g.w = Td * fmaf(mi.x - b0, r0, fmaf(mi.y - b1, r1, (mi.z - b2) * r2));
-                        scatter_pp<SPARSE>(G, SPARSE ? slots + (size_t)d * hw : nullptr, (unsigned)d, hw, H, W, t, g,
-                                           ng);
+                    const float gc = Td * mi.w;
+                    float4 g;
+                    g.x = gc * r0;
+                    g.y = gc * r1;
+                    g.z = gc * r2;
+                    g.w = Td * fmaf(mi.x - b0, r0, fmaf(mi.y - b1, r1, (mi.z - b2) * r2));
+                    if (fast) {  // the taps are formed again: keeping them costs registers, and warps
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                        rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W, t.fx,
+                                              t.fy, g, ng);
+                    } else {
+                        const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
+                        if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);
                     }
                 }
                 const float om = 1.f - mi.w;
@@ -308,71 +336,56 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
             }
         }
     }
-    if (LOSS) {
+    // loss: one partial a tile, from the tile's first warp
+    const int tiles_x = (W + sh.tile_x - 1) / sh.tile_x;
+    if (LOSS && pc.g == 0 && pc.tile < sh.tiles && pc.tx < tiles_x) {
         lsum = rl_warp_sum(lsum);
-        if (pc.lane == 0) red[pc.g] = lsum;
-        __syncthreads();
-        float blk = 0.f;
-        if (threadIdx.x == 0)
-            for (int i = 0; i < kGroups; ++i) blk += red[i];
-        __syncthreads();
-        rl_loss_epilogue(blk, partials, bid, nblocks, loss_out, counter, loss_scale, threadIdx.x, kGroups * kPix,
-                         red);
+        const unsigned part = ((unsigned)pc.ty * (unsigned)tiles_x + (unsigned)pc.tx) * (unsigned)views.n +
+                              (unsigned)pc.view;
+        if (pc.lane == 0 && RL_IN(part, nparts)) partials[part] = lsum;
     }
 }
 
-template <typename Tm, int C, int kGroups, bool SPARSE, bool LOSS, bool ANCH>
-__global__ void __launch_bounds__(kGroups * kPix, C <= 4 ? 1024 / (kGroups * kPix) : 1)
-k_grad_pp(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views, int tiles_x,
+template <typename Tm, bool FULL, bool SPARSE, bool LOSS, bool ANCH>
+__global__ void __launch_bounds__(kMaxWarps * kPix, 2)
+k_grad_pp(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views, PPShape sh,
           const float* __restrict__ images, int img_level, const float* __restrict__ grad_out,
           const uint8_t* __restrict__ slots, float* __restrict__ G, float inv_n, float* __restrict__ partials,
-          float* __restrict__ loss_out, unsigned* __restrict__ counter, float loss_scale) {
-    __shared__ float4 xch[kGroups][kPix];
-    __shared__ float red[kGroups];
-    grad_pp_tile<Tm, C, kGroups, SPARSE, LOSS, ANCH>(M, D, H, W, views, pixel_coord(H, W), images, img_level, grad_out,
-                                               slots, G, inv_n, partials,
-                                               blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
-                                               gridDim.x * gridDim.y * gridDim.z, loss_out, counter, loss_scale, xch,
-                                               red);
+          unsigned nparts) {
+    // grid (views, blocks_x, tiles_y): the views of a tile run together and share M in L2
+    grad_pp_tile<Tm, FULL, SPARSE, LOSS, ANCH>(M, D, H, W, views,
+                                               pp_pos(H, W, blockIdx.x, blockIdx.y, blockIdx.z, sh), sh, blockIdx.y,
+                                               images, img_level, grad_out, slots, G, inv_n, partials, nparts);
 }
 
-// Batched gradient, plane-parallel family: one persistent launch of 8-warp blocks walks the
-// gradient units of the batch table's items that take this family (a unit is one 16 x 2 tile of
-// one view of one item, in the order of k_grad_pp's grid; planes per thread from the item's D),
-// each item with its own loss epilogue over its own units.
+// Batched gradient, plane-parallel family: one persistent launch of 16-warp blocks walks the
+// gradient units of the batch table's items that take this family (a unit is one block's tiles of
+// one view of one item).
 template <typename Tm>
-__global__ void __launch_bounds__(8 * kPix, 3)
+__global__ void __launch_bounds__(kMaxWarps * kPix, 2)
 k_grad_pp_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restrict__ items) {
-    __shared__ float4 xch[8][kPix];
-    __shared__ float red[8];
     const unsigned n = hdr->n, total = hdr->pp_units;
     if (hdr->dtype != (std::is_same<Tm, float>::value ? (unsigned)RL_F32 : (unsigned)RL_BF16)) return;
     __shared__ unsigned next_slot;
     for (unsigned u = rl_batch_next(hdr, 2, &next_slot); u < total; u = rl_batch_next(hdr, 2, &next_slot)) {
         const RLBatchItem& it = items[rl_batch_find(items, n, u, &RLBatchItem::pp_begin)];
         const unsigned local = u - it.pp_begin;
-        const unsigned view = local % (unsigned)it.N, tile = local / (unsigned)it.N;
+        const unsigned view = local % (unsigned)it.N, block = local / (unsigned)it.N;
         const int h = it.H >> it.level, w = it.W >> it.level;
-        const PixelCoord pc =
-            pixel_coord_at(h, w, (int)view, (int)(tile % it.pp_tiles_x), (int)(tile / it.pp_tiles_x));
+        const int bx = (int)(block % it.pp_tiles_x), by = (int)(block / it.pp_tiles_x);
+        const PPShape sh = grad_pp_shape(it.D, h, w, kMaxWarps);
         const Tm* Ml = static_cast<const Tm*>(it.Ml);
-#define RL_PPB(CC, A) grad_pp_tile<Tm, CC, 8, true, true, A>(Ml, it.D, h, w, it.views, pc,                       \
-                                                             it.level ? it.Il : it.images, 0,                       \
-                                                             nullptr, it.slots, it.G, it.inv_n, it.partials, local, \
-                                                             it.pp_units, it.loss_out, it.counter, it.loss_scale,   \
-                                                             xch, red)
-        const int c = (it.D + 7) / 8;
-        if (it.views.anchored) {
-            if (c <= 1) RL_PPB(1, true);
-            else if (c <= 2) RL_PPB(2, true);
-            else if (c <= 4) RL_PPB(4, true);
-            else RL_PPB(8, true);
-        } else {
-            if (c <= 1) RL_PPB(1, false);
-            else if (c <= 2) RL_PPB(2, false);
-            else if (c <= 4) RL_PPB(4, false);
-            else RL_PPB(8, false);
+        PPPos pc = pp_pos(h, w, (int)view, bx, by, sh);
+        if (pc.tile >= sh.tiles) {  // a warp without a tile: a chunk of the first one, used by none
+            pc.tx = bx * sh.tiles;
+            pc.g = 0;
+            pc.G = 1;
         }
+#define RL_PPB(A) grad_pp_tile<Tm, false, true, true, A>(Ml, it.D, h, w, it.views, pc, sh, bx,                  \
+                                                           it.level ? it.Il : it.images, 0, nullptr, it.slots,   \
+                                                           it.G, it.inv_n, it.partials, it.parts)
+        if (it.views.anchored) RL_PPB(true);
+        else RL_PPB(false);
 #undef RL_PPB
         __syncthreads();  // the exchange buffers are reused by the next unit
     }
@@ -384,47 +397,26 @@ int chunk_for(int D, int G) {
     return c <= 1 ? 1 : c <= 2 ? 2 : c <= 4 ? 4 : 8;
 }
 
-// Warps per block: 8 (measured faster than 4 at D = 32 despite the chunk combination being
-// amortised over fewer planes); kernel path 4 forces 4 where D <= 32 (at most 8 planes per
+// Warps per block of the render: 8 (measured faster than 4 at D = 32 despite the chunk combination
+// being amortised over fewer planes); kernel path 4 forces 4 where D <= 32 (at most 8 planes per
 // thread).
 int groups_for(int D, int path) {
     return (path == 4 && D <= 32) ? 4 : 8;
 }
 
 template <typename Tm, bool SPARSE, bool LOSS>
-void launch_grad_pp_t(int G, int C, const void* M, int D, int H, int W, const RLViews& views, int tiles_x, dim3 grid,
-                      const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G_,
-                      float inv_n, float* partials, float* loss_out, unsigned* counter, float loss_scale,
-                      cudaStream_t s) {
-#define RL_PP_ARGS (const Tm*)M, D, H, W, views, tiles_x, images, img_level, grad_out, slots, G_, inv_n, partials, \
-                   loss_out, counter, loss_scale
-#define RL_PP_LAUNCH(CC, GG) k_grad_pp<Tm, CC, GG, SPARSE, LOSS, false><<<grid, GG * kPix, 0, s>>>(RL_PP_ARGS)
-#define RL_PP_LAUNCH_A(CC) k_grad_pp<Tm, CC, 8, SPARSE, LOSS, true><<<grid, 8 * kPix, 0, s>>>(RL_PP_ARGS)
-    if (views.anchored) {  // 8 warps a block (the 4-warp option keeps the FP32 coordinates only)
-        switch (C) {
-            case 1: RL_PP_LAUNCH_A(1); break;
-            case 2: RL_PP_LAUNCH_A(2); break;
-            case 4: RL_PP_LAUNCH_A(4); break;
-            default: RL_PP_LAUNCH_A(8); break;
-        }
-    } else if (G == 4) {
-        switch (C) {
-            case 1: RL_PP_LAUNCH(1, 4); break;
-            case 2: RL_PP_LAUNCH(2, 4); break;
-            case 4: RL_PP_LAUNCH(4, 4); break;
-            default: RL_PP_LAUNCH(8, 4); break;
-        }
-    } else {
-        switch (C) {
-            case 1: RL_PP_LAUNCH(1, 8); break;
-            case 2: RL_PP_LAUNCH(2, 8); break;
-            case 4: RL_PP_LAUNCH(4, 8); break;
-            default: RL_PP_LAUNCH(8, 8); break;
-        }
-    }
-#undef RL_PP_LAUNCH_A
+void launch_grad_pp_t(const PPShape sh, const void* M, int D, int H, int W, const RLViews& views, const float* images,
+                      int img_level, const float* grad_out, const uint8_t* slots, float* G, float inv_n,
+                      float* partials, unsigned nparts, cudaStream_t s) {
+    const int per = sh.tile_x * sh.tiles, rows = kPix / sh.tile_x;
+    const dim3 grid((unsigned)views.n, (unsigned)((W + per - 1) / per), (unsigned)((H + rows - 1) / rows));
+    const unsigned threads = (unsigned)(sh.G * sh.tiles * kPix);
+#define RL_PP_LAUNCH(FULL, A)                                                                                       \
+    k_grad_pp<Tm, FULL, SPARSE, LOSS, A><<<grid, threads, 0, s>>>((const Tm*)M, D, H, W, views, sh, images,        \
+                                                                  img_level, grad_out, slots, G, inv_n, partials, nparts)
+    if (D % kChunk == 0) { if (views.anchored) RL_PP_LAUNCH(true, true); else RL_PP_LAUNCH(true, false); }
+    else { if (views.anchored) RL_PP_LAUNCH(false, true); else RL_PP_LAUNCH(false, false); }
 #undef RL_PP_LAUNCH
-#undef RL_PP_ARGS
 }
 
 template <typename Tm>
@@ -461,33 +453,36 @@ void launch_render_pp_t(int G, int C, const void* M, int D, int H, int W, const 
 
 }  // namespace
 
+// Tiles of a gradient launch over all views: the loss partials it writes.
 size_t rl_grad_pp_num_blocks(int H, int W, int N) {
-    return (size_t)((W + kTX - 1) / kTX) * ((H + kTY - 1) / kTY) * N;
+    const int tx = grad_pp_tile_x(H, W), ty = kPix / tx;
+    return (size_t)((W + tx - 1) / tx) * ((H + ty - 1) / ty) * N;
 }
 
 rl_status rl_launch_grad_pp(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                             const float* images, int img_level, const float* grad_out, const uint8_t* slots,
-                            float* G_out, float inv_n, float* partials, int* nblocks, cudaStream_t s,
-                            float* loss_out, unsigned* counter, float loss_scale) {
-    const int tiles_x = (W + kTX - 1) / kTX;
-    const dim3 grid((unsigned)views.n, (unsigned)tiles_x, (unsigned)((H + kTY - 1) / kTY));
-    if (nblocks) *nblocks = (int)rl_grad_pp_num_blocks(H, W, views.n);
-    const int G = views.anchored ? 8 : groups_for(D, rl_kernel_path_setting());
-    const int C = chunk_for(D, G);
+                            float* G_out, float inv_n, float* partials, int* nblocks, cudaStream_t s) {
+    // kernel path 4 asks for narrower blocks
+    const PPShape sh = grad_pp_shape(D, H, W, rl_kernel_path_setting() == 4 ? 4 : 8);
+    const unsigned nparts = (unsigned)rl_grad_pp_num_blocks(H, W, views.n);
+    if (nblocks) *nblocks = (int)nparts;
     const bool sparse = slots != nullptr;
     const char* name = dt == RL_F32 ? (sparse ? "grad_sparse_f32" : "grad_dense_f32")
                                     : (sparse ? "grad_sparse_bf16" : "grad_dense_bf16");
     RLTraceScope ts(name, s);
 #define RL_CASE(TM, SP, LS) \
-    launch_grad_pp_t<TM, SP, LS>(G, C, M, D, H, W, views, tiles_x, grid, images, img_level, grad_out, slots, G_out, \
-                                 inv_n, partials, loss_out, counter, loss_scale, s)
-    if (dt == RL_F32) {
-        if (sparse) { if (mode_loss) RL_CASE(float, true, true); else RL_CASE(float, true, false); }
-        else        { if (mode_loss) RL_CASE(float, false, true); else RL_CASE(float, false, false); }
-    } else {
-        if (sparse) { if (mode_loss) RL_CASE(__nv_bfloat16, true, true); else RL_CASE(__nv_bfloat16, true, false); }
-        else        { if (mode_loss) RL_CASE(__nv_bfloat16, false, true); else RL_CASE(__nv_bfloat16, false, false); }
-    }
+    launch_grad_pp_t<TM, SP, LS>(sh, M, D, H, W, views, images, img_level, grad_out, slots, G_out, inv_n, partials, \
+                                 nparts, s)
+    // a slot map comes with the loss mode only
+#define RL_KIND(TM)                                                                               \
+    do {                                                                                          \
+        if (slots) RL_CASE(TM, true, true);                                                      \
+        else if (mode_loss) RL_CASE(TM, false, true);                                            \
+        else RL_CASE(TM, false, false);                                                          \
+    } while (0)
+    if (dt == RL_F32) RL_KIND(float);
+    else RL_KIND(__nv_bfloat16);
+#undef RL_KIND
 #undef RL_CASE
     return rl_check_launch("grad_pp");
 }
@@ -508,20 +503,27 @@ rl_status rl_launch_render_pp(const void* M, rl_dtype dt, int D, int H, int W, c
     return rl_check_launch("render_pp");
 }
 
-unsigned rl_grad_pp_tiles_x(int w) { return (unsigned)((w + kTX - 1) / kTX); }
-unsigned rl_grad_pp_tiles_y(int h) { return (unsigned)((h + kTY - 1) / kTY); }
+unsigned rl_grad_pp_tiles_x(int h, int w, int D) {
+    const PPShape sh = grad_pp_shape(D, h, w, kMaxWarps);
+    const int per = sh.tile_x * sh.tiles;
+    return (unsigned)((w + per - 1) / per);
+}
+unsigned rl_grad_pp_tiles_y(int h, int w) {
+    const int rows = kPix / grad_pp_tile_x(h, w);
+    return (unsigned)((h + rows - 1) / rows);
+}
 
 rl_status rl_launch_grad_pp_batch(const void* table, rl_dtype dt, cudaStream_t s) {
     const RLBatchHeader* hdr = static_cast<const RLBatchHeader*>(table);
     const RLBatchItem* items = rl_batch_items(table);
-    const int grid = dt == RL_F32 ? rl_persistent_grid<k_grad_pp_batch<float>>(8 * kPix, 0)
-                                  : rl_persistent_grid<k_grad_pp_batch<__nv_bfloat16>>(8 * kPix, 0);
+    const int grid = dt == RL_F32 ? rl_persistent_grid<k_grad_pp_batch<float>>(kMaxWarps * kPix, 0)
+                                  : rl_persistent_grid<k_grad_pp_batch<__nv_bfloat16>>(kMaxWarps * kPix, 0);
     if (dt == RL_F32) {
         RLTraceScope ts("grad_pp_batch_f32", s);
-        k_grad_pp_batch<float><<<grid, 8 * kPix, 0, s>>>(hdr, items);
+        k_grad_pp_batch<float><<<grid, kMaxWarps * kPix, 0, s>>>(hdr, items);
     } else {
         RLTraceScope ts("grad_pp_batch_bf16", s);
-        k_grad_pp_batch<__nv_bfloat16><<<grid, 8 * kPix, 0, s>>>(hdr, items);
+        k_grad_pp_batch<__nv_bfloat16><<<grid, kMaxWarps * kPix, 0, s>>>(hdr, items);
     }
     return rl_check_launch("grad_pp_batch");
 }

@@ -118,7 +118,6 @@ struct RLBatchItem {
     uint8_t* slots;          // slot map [D][h][w]
     float* G;                // compact gradient [k][h][w][4]
     float* partials;         // loss partials, one per gradient unit
-    unsigned* counter;       // last-block counter of the loss epilogue
     float* loss_out;         // device [1] or NULL
     float* Il;               // level-l source images [N][h][w][3] (levels >= 1; written by the selection)
     int D, H, W, level, k, mode, clamp01, N;
@@ -126,7 +125,8 @@ struct RLBatchItem {
     unsigned sel_begin, sel_units;    // first unit and unit count of each stage
     unsigned grad_begin, grad_units, grad_tiles_x;   // gather family (units 0 for the other items)
     unsigned pp_begin, pp_units, pp_tiles_x;         // plane-parallel family (units 0 for the others)
-    unsigned upd_begin, upd_units, upd_tiles_x, pad;
+    unsigned upd_begin, upd_units, upd_tiles_x;
+    unsigned parts;          // loss partials of the item's gradient
     RLViews views;           // level-l warp parameters of the N views and the plane inverse depths
 };
 
@@ -506,41 +506,194 @@ __device__ __forceinline__ float4 rl_sample_fast(const Tm* __restrict__ plane, i
 // Slot-map value of a voxel that the selection did not keep.
 #define RL_SLOT_NONE 0xFF
 
+// ------------------------------------------------------------------ fast samples
+//
+// Fast coordinates of a sample known to lie inside the plane: the floor comes from an addition
+// rounded towards minus infinity to a multiple of one (exact for |s| < 2^22), whose mantissa is
+// also the integer part, so that a sample needs no conversion instruction and one multiply-add
+// forms its voxel index.  Same values as rl_taps / rl_anchor_taps.
+#define RL_FLOOR_MAGIC 12582912.f  // 1.5 * 2^23
+#define RL_FLOOR_BITS 0x4B400000u
+#define RL_FAST_EXTENT (1 << 20)       // image sides for which the fast coordinates are exact
+
+struct RLFastTap {
+    unsigned idx;  // voxel of the top-left tap within its plane
+    float fx, fy;
+};
+
+__device__ __forceinline__ unsigned rl_fast_base(int qx, int qy, int W) {
+    return (unsigned)qy * (unsigned)W + (unsigned)qx - RL_FLOOR_BITS * ((unsigned)W + 1u);
+}
+
+template <bool ANCH>
+__device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const RLAnchor& A, int d, float rho,
+                                            unsigned base, int W) {
+    float sx, sy;
+    if constexpr (ANCH) {
+        const RLPlaneK k = A.k[d];
+        sx = k.fx + fmaf(rho, w.w.dbx, w.w.dax);
+        sy = k.fy + fmaf(rho, w.w.dby, w.w.day);
+        base += (unsigned)(k.iy * W + k.ix);
+    } else {
+        sx = fmaf(rho, w.w.bx, w.w.ax);
+        sy = fmaf(rho, w.w.by, w.w.ay);
+    }
+    const float tx = __fadd_rd(sx, RL_FLOOR_MAGIC), ty = __fadd_rd(sy, RL_FLOOR_MAGIC);
+    RLFastTap t;
+    t.fx = sx - (tx - RL_FLOOR_MAGIC);
+    t.fy = sy - (ty - RL_FLOOR_MAGIC);
+    t.idx = base + __float_as_uint(ty) * (unsigned)W + __float_as_uint(tx);
+    return t;
+}
+
+// True when the samples of every plane in [d_lo, d_hi] lie inside the plane, at least a pixel from
+// its border, and the planes are met in front of the view: position and depth factor are linear in
+// the plane's inverse depth, so the two end planes bound the others.  The pixel of margin covers
+// the rounding.
+template <bool ANCH>
+__device__ __forceinline__ bool rl_chunk_inside(const RLPixWarp<ANCH>& w, const RLAnchor& A, const RLViews& views,
+                                                int d_lo, int d_hi, int qx, int qy, int H, int W) {
+    const float rho0 = views.rho[d_lo], rho1 = views.rho[d_hi];
+    float x0, y0, x1, y1;
+    bool ok;
+    if constexpr (ANCH) {
+        const RLPlaneK a = A.k[d_lo], b = A.k[d_hi];
+        ok = w.w.ok && a.ix != RL_PLANE_NONE && b.ix != RL_PLANE_NONE;
+        x0 = (float)(qx + a.ix) + (a.fx + fmaf(rho0, w.w.dbx, w.w.dax));
+        y0 = (float)(qy + a.iy) + (a.fy + fmaf(rho0, w.w.dby, w.w.day));
+        x1 = (float)(qx + b.ix) + (b.fx + fmaf(rho1, w.w.dbx, w.w.dax));
+        y1 = (float)(qy + b.iy) + (b.fy + fmaf(rho1, w.w.dby, w.w.day));
+    } else {
+        ok = w.w.dir_ok && fmaf(-rho0, w.w.cz, 1.0f) > 0.0f && fmaf(-rho1, w.w.cz, 1.0f) > 0.0f;
+        x0 = (float)qx + fmaf(rho0, w.w.bx, w.w.ax);
+        y0 = (float)qy + fmaf(rho0, w.w.by, w.w.ay);
+        x1 = (float)qx + fmaf(rho1, w.w.bx, w.w.ax);
+        y1 = (float)qy + fmaf(rho1, w.w.by, w.w.ay);
+    }
+    // a NaN position fails the comparisons; sides beyond RL_FAST_EXTENT take the general path
+    return ok && (H | W) < RL_FAST_EXTENT && fminf(x0, x1) >= 1.f && fmaxf(x0, x1) < (float)(W - 2) &&
+           fminf(y0, y1) >= 1.f && fmaxf(y0, y1) < (float)(H - 2);
+}
+
+// The four taps of a sample blended with packed FP32x2 FMAs (the order of rl_sample).
+__device__ __forceinline__ float4 rl_blend(const float4& v00, const float4& v10, const float4& v01, const float4& v11,
+                                           float fx, float fy) {
+    const float gx = 1.f - fx, gy = 1.f - fy;
+    const float w00 = gx * gy, w10 = fx * gy, w01 = gx * fy, w11 = fx * fy;
+    float2 lo = __fmul2_rn(make_float2(w00, w00), make_float2(v00.x, v00.y));
+    float2 hi = __fmul2_rn(make_float2(w00, w00), make_float2(v00.z, v00.w));
+    lo = __ffma2_rn(make_float2(w10, w10), make_float2(v10.x, v10.y), lo);
+    hi = __ffma2_rn(make_float2(w10, w10), make_float2(v10.z, v10.w), hi);
+    lo = __ffma2_rn(make_float2(w01, w01), make_float2(v01.x, v01.y), lo);
+    hi = __ffma2_rn(make_float2(w01, w01), make_float2(v01.z, v01.w), hi);
+    lo = __ffma2_rn(make_float2(w11, w11), make_float2(v11.x, v11.y), lo);
+    hi = __ffma2_rn(make_float2(w11, w11), make_float2(v11.z, v11.w), hi);
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+// Sample inside the plane: voxel e of the MPI is the top-left tap.
+template <typename Tm>
+__device__ __forceinline__ float4 rl_sample_at(const Tm* __restrict__ M, unsigned e, int W, float fx, float fy) {
+    const Tm* p = M + (size_t)e * 4u;
+    const Tm* q = M + (size_t)(e + (unsigned)W) * 4u;
+    return rl_blend(RLStore<Tm>::load4(p), RLStore<Tm>::load4(p + 4), RLStore<Tm>::load4(q), RLStore<Tm>::load4(q + 4),
+                    fx, fy);
+}
+
+// Adds wt (gl, gh) to one voxel of the gradient.
+__device__ __forceinline__ void rl_add_tap(float4* __restrict__ G4, unsigned at, float wt, float2 gl, float2 gh) {
+    const float2 a = __fmul2_rn(make_float2(wt, wt), gl), b = __fmul2_rn(make_float2(wt, wt), gh);
+    atomicAdd(G4 + at, make_float4(a.x, a.y, b.x, b.y));
+}
+
+// The slots of the four taps (00, 10, 01, 11, a byte each) of a sample inside the plane whose
+// top-left tap is voxel e of the MPI: loaded with the sample, ahead of the scatter that needs them.
+__device__ __forceinline__ unsigned rl_slot_word(const uint8_t* __restrict__ slots, unsigned e, int W) {
+    const uint8_t* p = slots + e;
+    const uint8_t* q = p + W;
+    return (unsigned)__ldg(p) | (unsigned)__ldg(p + 1) << 8 | (unsigned)__ldg(q) << 16 | (unsigned)__ldg(q + 1) << 24;
+}
+
+// Bilinear transpose of the gradient g of a sample inside the plane: top-left tap p of its plane,
+// voxel e of the MPI.  SPARSE: only into the taps that have a slot in the compact gradient.
+template <bool SPARSE>
+__device__ __forceinline__ void rl_scatter_at(float* __restrict__ G, unsigned word, unsigned d, unsigned p, unsigned e,
+                                              unsigned hw, int W, float fx, float fy, float4 g, unsigned ng) {
+    float4* G4 = reinterpret_cast<float4*>(G);
+    const float gx = 1.f - fx, gy = 1.f - fy;
+    const float2 gl = make_float2(g.x, g.y), gh = make_float2(g.z, g.w);
+    if constexpr (SPARSE) {
+        if (word == 0xFFFFFFFFu) return;
+        const unsigned s00 = word & 255u, s10 = (word >> 8) & 255u, s01 = (word >> 16) & 255u, s11 = word >> 24;
+        if (s00 != RL_SLOT_NONE && RL_IN(s00, ng)) rl_add_tap(G4, s00 * hw + p, gx * gy, gl, gh);
+        if (s10 != RL_SLOT_NONE && RL_IN(s10, ng)) rl_add_tap(G4, s10 * hw + p + 1u, fx * gy, gl, gh);
+        if (s01 != RL_SLOT_NONE && RL_IN(s01, ng)) rl_add_tap(G4, s01 * hw + p + (unsigned)W, gx * fy, gl, gh);
+        if (s11 != RL_SLOT_NONE && RL_IN(s11, ng)) rl_add_tap(G4, s11 * hw + p + (unsigned)W + 1u, fx * fy, gl, gh);
+    } else {
+        if (!RL_IN(d, ng)) return;
+        rl_add_tap(G4, e, gx * gy, gl, gh);
+        rl_add_tap(G4, e + 1u, fx * gy, gl, gh);
+        rl_add_tap(G4, e + (unsigned)W, gx * fy, gl, gh);
+        rl_add_tap(G4, e + (unsigned)W + 1u, fx * fy, gl, gh);
+    }
+}
+
+template <bool SPARSE>
+__device__ __forceinline__ void rl_scatter_tap(float* __restrict__ G, const uint8_t* __restrict__ slots, unsigned d,
+                                               unsigned hw, int H, int W, int x, int y, float wt, float4 g,
+                                               unsigned ng) {
+    if ((unsigned)x >= (unsigned)W || (unsigned)y >= (unsigned)H) return;
+    const unsigned pix = (unsigned)(y * W + x);
+    const unsigned slot = SPARSE ? (unsigned)__ldg(slots + (d * hw + pix)) : d;
+    if ((SPARSE && slot == RL_SLOT_NONE) || !RL_IN(slot, ng)) return;
+    rl_add_tap(reinterpret_cast<float4*>(G), slot * hw + pix, wt, make_float2(g.x, g.y), make_float2(g.z, g.w));
+}
+
+// The same transpose with each tap tested against the plane.
+template <bool SPARSE>
+__device__ __forceinline__ void rl_scatter(float* __restrict__ G, const uint8_t* __restrict__ slots, unsigned d,
+                                           unsigned hw, int H, int W, const RLTaps& t, float4 g, unsigned ng) {
+    const float gx = 1.f - t.fx, gy = 1.f - t.fy;
+    rl_scatter_tap<SPARSE>(G, slots, d, hw, H, W, t.x0, t.y0, gx * gy, g, ng);
+    rl_scatter_tap<SPARSE>(G, slots, d, hw, H, W, t.x0 + 1, t.y0, t.fx * gy, g, ng);
+    rl_scatter_tap<SPARSE>(G, slots, d, hw, H, W, t.x0, t.y0 + 1, gx * t.fy, g, ng);
+    rl_scatter_tap<SPARSE>(G, slots, d, hw, H, W, t.x0 + 1, t.y0 + 1, t.fx * t.fy, g, ng);
+}
+
 __device__ __forceinline__ float rl_warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// Loss epilogue shared by the gradient kernels.  Thread `tid` 0 of every block passes the
-// block's partial sum `s`; it is stored at partials[bid].  When out != NULL the last block
-// to finish (counted on *counter, which must be 0 at launch and is reset to 0 here) adds
-// all nblocks partials in index order -- a fixed order, so the loss is deterministic -- and
-// writes out[0] = sum * scale.  `red` is shared scratch of nthreads / 32 floats.
-__device__ __forceinline__ void rl_loss_epilogue(float s, float* __restrict__ partials, unsigned bid, unsigned nblocks,
-                                                 float* __restrict__ out, unsigned* __restrict__ counter, float scale,
-                                                 int tid, int nthreads, float* red) {
-    __shared__ int rl_am_last;
-    if (tid == 0) {
-        if (RL_IN(bid, nblocks)) partials[bid] = s;
-        rl_am_last = 0;
-        if (out) {
-            __threadfence();
-            rl_am_last = atomicAdd(counter, 1u) == nblocks - 1;
-        }
+// One compensated addition (Kahan): s + c carries the running sum of FP32 values to about FP64.
+__device__ __forceinline__ void rl_kahan_add(float& s, float& c, float v) {
+    const float y = v - c, t = s + y;
+    c = (t - s) - y;
+    s = t;
+}
+
+// Sum of the n loss partials at `partials` (16-byte aligned) by one block, in an order fixed by n and
+// the block's size, so the loss is deterministic.  The total is returned to thread 0; `red` is shared
+// scratch of nthreads / 32 floats.
+__device__ __forceinline__ float rl_partials_sum(const float* __restrict__ partials, unsigned n, int tid, int nthreads,
+                                                 float* red) {
+    float a[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
+    const unsigned n4 = n / 4;
+#pragma unroll 8
+    for (unsigned i = tid; i < n4; i += nthreads) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(partials) + i);
+        rl_kahan_add(a[0], c[0], v.x);
+        rl_kahan_add(a[1], c[1], v.y);
+        rl_kahan_add(a[2], c[2], v.z);
+        rl_kahan_add(a[3], c[3], v.w);
     }
-    __syncthreads();
-    if (!rl_am_last) return;
-    __threadfence();
-    float acc = 0.f;
-    for (unsigned i = tid; i < nblocks; i += nthreads) acc += __ldcg(partials + i);
-    acc = rl_warp_sum(acc);
+    if (tid < (int)(n & 3u)) rl_kahan_add(a[0], c[0], __ldcg(partials + n4 * 4 + tid));
+    const float acc = rl_warp_sum((a[0] + a[1]) + (a[2] + a[3]));
     if ((tid & 31) == 0) red[tid >> 5] = acc;
     __syncthreads();
-    if (tid == 0) {
-        float total = 0.f;
+    float total = 0.f;
+    if (tid == 0)
         for (int wi = 0; wi < nthreads / 32; ++wi) total += red[wi];
-        out[0] = total * scale;
-        *counter = 0u;
-    }
+    return total;
 }

@@ -27,11 +27,21 @@ struct RLTraceScope {
 // Device status word (bit RL_DEVFLAG_TIMEOUT: a bounded wait gave up); address on the
 // current device, or NULL if it cannot be resolved.
 unsigned int* rl_device_status_ptr();
-// Warp-kernel family for a launch over H x W pixels of n views: 2 per-pixel gather,
-// 3 plane-parallel.  The automatic setting picks plane-parallel for launches of fewer than
-// 2^19 pixel-views (coarse pyramid levels, small requests), where per-pixel threads are too
-// few to hide gather latency, and per-pixel gather otherwise.
+// Warp-kernel family of a render over H x W pixels of n views: 2 per-pixel gather, 3
+// plane-parallel.  The automatic setting picks plane-parallel for launches of fewer than
+// 2^19 pixel-views (small views), where per-pixel threads are too few to hide gather latency,
+// and per-pixel gather otherwise.
 int rl_kernel_path(int H, int W, int nviews);
+// The same for the gradient.  Automatic: plane-parallel, which gathers each sample once (512x384,
+// 4 views, BF16: 206 against 246 us at D = 32, 442 against 465 us at D = 64; 64x48, 2 views, D = 32:
+// 13 against 51 us), except launches of 2^19 pixel-views or more with anchored coordinates: a
+// plane-parallel block repeats the FP64 set-up of the anchors for every 32 pixels, a per-pixel one
+// for every 128 (1024x768, 4 views, D = 64, BF16: 2507 against 1710 us; at 2^18.6 pixel-views equal).
+int rl_grad_path(int H, int W, int nviews, bool anchored);
+// The gradient family of a batched step of so many pixel-views in all: per-pixel gather, whose long
+// units hide the cost of fetching them (eight requests of 2 to 50 M samples: 2484 us against 3475 us
+// plane-parallel), unless the whole batch is too small to fill the device with them.
+int rl_batch_grad_path(long long pixel_views);
 // The raw process-wide setting of reallife_set_kernel_path (0, 2 to 5).
 int rl_kernel_path_setting();
 
@@ -61,21 +71,17 @@ rl_status rl_launch_warp_offsets(int D, int H, int W, const RLViews& views, floa
 
 // Fused warp + composite + residual + adjoint.  mode_loss: residual from images (full-res
 // images at level img_level, averaged on the fly) else from grad_out.  slots != NULL
-// (slot map [D][H][W], RL_SLOT_NONE where not kept): compact gradient [k][H][W][4]; else
+// (slot map [D][H][W], RL_SLOT_NONE where not kept; mode_loss only): compact gradient [k][H][W][4]; else
 // dense [D][H][W][4].  partials: one float per block
-// (loss mode); returns the number of blocks through *nblocks.  With loss_out != NULL the
-// last block also writes loss_out[0] = loss_scale * (sum of the partials), counting blocks
-// on *counter (0 at launch, left at 0).
+// (loss mode, 16-byte aligned); returns the number of blocks through *nblocks.
 rl_status rl_launch_grad(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                          const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G,
-                         float inv_n, float* partials, int* nblocks, cudaStream_t s, float* loss_out = nullptr,
-                         unsigned* counter = nullptr, float loss_scale = 0.f);
+                         float inv_n, float* partials, int* nblocks, cudaStream_t s);
 // Largest number of loss partials any gradient kernel family writes.
 size_t rl_grad_num_blocks(int H, int W, int N);
 rl_status rl_launch_grad_pp(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                             const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G,
-                            float inv_n, float* partials, int* nblocks, cudaStream_t s, float* loss_out,
-                            unsigned* counter, float loss_scale);
+                            float inv_n, float* partials, int* nblocks, cudaStream_t s);
 size_t rl_grad_pp_num_blocks(int H, int W, int N);
 rl_status rl_launch_render_pp(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, float* out,
                               cudaStream_t s);
@@ -85,24 +91,30 @@ rl_status rl_launch_loss_reduce(const float* partials, int n, float scale, float
 // Outputs (each optional): S [k][h][w], mask [h][w], slot map [D][h][w]; Gzero
 // [k][h][w][4] is zeroed.
 rl_status rl_launch_select(const void* M, rl_dtype dt, const float* keys, int D, int h, int w, int k, uint8_t* S,
-                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s,
-                           unsigned* counter_zero = nullptr, int mode = 0);
+                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, int mode = 0);
 // Level-l MPI Ml [D][H>>l][W>>l][4] = Down^l(M) (level >= 1) and the selection on it in one pass: outputs as
 // rl_launch_select without the mask, identical values.  With images and Il != NULL it also writes the
 // level-l source images Il [N][H>>l][W>>l][3] (2^l x 2^l means of images [N][H][W][3], formed exactly as
 // the gradient kernels form them on the fly), which the gradient then reads at img_level 0.
 rl_status rl_launch_pyramid_select(const void* M, rl_dtype dt, int D, int H, int W, int level, void* Ml, int k,
-                                   uint8_t* S, uint8_t* slots, float* Gzero, unsigned* counter_zero, int mode,
-                                   cudaStream_t s, const float* images = nullptr, int N = 0, float* Il = nullptr);
+                                   uint8_t* S, uint8_t* slots, float* Gzero, int mode, cudaStream_t s,
+                                   const float* images = nullptr, int N = 0, float* Il = nullptr);
 // Slot map [D][h][w] from a selection mask [h][w]: the kept planes of a pixel in ascending order
 // take slots 0 .. k-1; kept planes beyond the first k get no slot.
 rl_status rl_launch_mask_to_slots(const uint64_t* mask, int D, int k, int hw, uint8_t* slots, cudaStream_t s);
 rl_status rl_launch_downsample_f32(const float* x, int P, int H, int W, int C, int level, float* y,
                                    cudaStream_t s);
-// With Ml (level MPI) and lambda_s != 0 the sparsity prior joins the alpha step.
+// With Ml (level MPI) and lambda_s != 0 the sparsity prior joins the alpha step.  With loss.out the
+// first block also writes loss.out[0] = loss.scale * (sum of the loss.n partials) of the gradient.
+struct RLLossSum {
+    const float* partials = nullptr;  // 16-byte aligned
+    int n = 0;
+    float scale = 0.f;
+    float* out = nullptr;
+};
 rl_status rl_launch_update(void* M, rl_dtype dt, int D, int H, int W, int level, const uint8_t* S, const float* G,
                            int k, float lambda, int clamp01, cudaStream_t s, const void* Ml = nullptr,
-                           float lambda_s = 0.f);
+                           float lambda_s = 0.f, const RLLossSum& loss = RLLossSum());
 
 // Batched stages of one HSGD iteration over a batch table in device memory (header and items
 // of rl_common.cuh), each one persistent launch of one wave of resident blocks.  The gradient
@@ -114,8 +126,8 @@ rl_status rl_launch_grad_pp_batch(const void* table, rl_dtype dt, cudaStream_t s
 rl_status rl_launch_update_batch(const void* table, rl_dtype dt, cudaStream_t s);
 unsigned rl_grad_gather_tiles_x(int w);
 unsigned rl_grad_gather_tiles_y(int h);
-unsigned rl_grad_pp_tiles_x(int w);
-unsigned rl_grad_pp_tiles_y(int h);
+unsigned rl_grad_pp_tiles_x(int h, int w, int D);
+unsigned rl_grad_pp_tiles_y(int h, int w);
 
 // Blocks of a persistent launch of `kernel`: the resident blocks per SM on the current device
 // times its SMs (at least one); computed once per device and kernel instantiation.

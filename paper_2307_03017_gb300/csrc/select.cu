@@ -143,10 +143,9 @@ template <typename Tm, bool FROM_KEYS, int K>
 __global__ void __launch_bounds__(128)
 k_select(const Tm* __restrict__ M, const float* __restrict__ keys, int D, int h, int w, int k,
          uint8_t* __restrict__ S, uint64_t* __restrict__ mask_out, uint8_t* __restrict__ slots,
-         float* __restrict__ Gzero, unsigned* __restrict__ counter_zero, int mode) {
+         float* __restrict__ Gzero, int mode) {
     const long long hw = (long long)h * w;
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0 && counter_zero) *counter_zero = 0u;  // block counter of the loss epilogue that follows
     if (p >= hw) return;
     const uint64_t mk = select_mask<K, FROM_KEYS>(
         [&](int d) {
@@ -198,12 +197,11 @@ constexpr int kTile = 32;
 template <typename Tm, int K, int LOG>
 __device__ __forceinline__ void pyramid_select_tile(const Tm* __restrict__ M, int D, int H, int W, int level,
                                                     Tm* __restrict__ Ml, int k, uint8_t* __restrict__ S,
-                                                    uint8_t* __restrict__ slots, float* __restrict__ Gzero,
-                                                    unsigned* __restrict__ counter_zero, int mode, long long p0,
+                                                    uint8_t* __restrict__ slots, float* __restrict__ Gzero, int mode,
+                                                    long long p0,
                                                     float (*alpha)[kTile]) {
     const int h = H >> level, w = W >> level;
     const long long hw = (long long)h * w;
-    if (p0 == 0 && threadIdx.x == 0 && counter_zero) *counter_zero = 0u;
     // level 1: the loads of NB voxels (4 full-resolution voxels each) are issued together
     constexpr int NB = LOG == 1 ? 4 : 1;
     for (int i0 = threadIdx.x; i0 < D * kTile; i0 += NB * blockDim.x) {
@@ -290,12 +288,12 @@ __device__ __forceinline__ void level_image_means(const float* __restrict__ imag
 template <typename Tm, int K, int LOG>
 __global__ void __launch_bounds__(256)
 k_pyramid_select(const Tm* __restrict__ M, int D, int H, int W, int level, Tm* __restrict__ Ml, int k,
-                 uint8_t* __restrict__ S, uint8_t* __restrict__ slots, float* __restrict__ Gzero,
-                 unsigned* __restrict__ counter_zero, int mode, const float* __restrict__ images, int N,
+                 uint8_t* __restrict__ S, uint8_t* __restrict__ slots, float* __restrict__ Gzero, int mode,
+                 const float* __restrict__ images, int N,
                  float* __restrict__ Il) {
     __shared__ float alpha[RL_DEV_MAX_PLANES][kTile];
     if (Il) level_image_means<LOG>(images, N, H, W, level, Il, (long long)blockIdx.x * kTile);
-    pyramid_select_tile<Tm, K, LOG>(M, D, H, W, level, Ml, k, S, slots, Gzero, counter_zero, mode,
+    pyramid_select_tile<Tm, K, LOG>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode,
                                     (long long)blockIdx.x * kTile, alpha);
 }
 
@@ -316,10 +314,10 @@ __device__ __noinline__ uint64_t select_l0_ranked(const Tm* __restrict__ M, long
 template <typename Tm, int LOG>
 __device__ __noinline__ void pyramid_select_tile_ranked(const Tm* __restrict__ M, int D, int H, int W, int level,
                                                         Tm* __restrict__ Ml, int k, uint8_t* __restrict__ S,
-                                                        uint8_t* __restrict__ slots, float* __restrict__ Gzero,
-                                                        unsigned* __restrict__ counter_zero, int mode, long long p0,
+                                                        uint8_t* __restrict__ slots, float* __restrict__ Gzero, int mode,
+                                                    long long p0,
                                                         float (*alpha)[kTile]) {
-    pyramid_select_tile<Tm, 64, LOG>(M, D, H, W, level, Ml, k, S, slots, Gzero, counter_zero, mode, p0, alpha);
+    pyramid_select_tile<Tm, 64, LOG>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, p0, alpha);
 }
 
 template <typename Tm>
@@ -340,7 +338,6 @@ k_select_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
         if (it.level == 0) {
             const long long hw = (long long)it.H * it.W;
             const long long p = local * 256 + threadIdx.x;
-            if (p == 0) *it.counter = 0u;  // block counter of the loss epilogue that follows
             if (p < hw) {
                 const uint64_t mk =
                     ranked ? select_l0_ranked<Tm>(M, hw, p, it.D, it.k, it.mode)
@@ -352,11 +349,11 @@ k_select_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
             Tm* Ml = static_cast<Tm*>(it.Ml);
 #define RL_PSB(LL)                                                                                                 \
     if (ranked)                                                                                                    \
-        pyramid_select_tile_ranked<Tm, LL>(M, it.D, it.H, it.W, it.level, Ml, it.k, it.S, it.slots, it.G, it.counter, \
-                                           it.mode, local * kTile, alpha);                                         \
+        pyramid_select_tile_ranked<Tm, LL>(M, it.D, it.H, it.W, it.level, Ml, it.k, it.S, it.slots, it.G, it.mode, \
+                                           local * kTile, alpha);                                                  \
     else                                                                                                           \
-        pyramid_select_tile<Tm, 8, LL>(M, it.D, it.H, it.W, it.level, Ml, it.k, it.S, it.slots, it.G, it.counter,     \
-                                       it.mode, local * kTile, alpha)
+        pyramid_select_tile<Tm, 8, LL>(M, it.D, it.H, it.W, it.level, Ml, it.k, it.S, it.slots, it.G, it.mode,   \
+                                       local * kTile, alpha)
             if (it.level == 1) { level_image_means<1>(it.images, it.N, it.H, it.W, 1, it.Il, local * kTile); RL_PSB(1); }
             else if (it.level == 2) { level_image_means<2>(it.images, it.N, it.H, it.W, 2, it.Il, local * kTile); RL_PSB(2); }
             else { level_image_means<-1>(it.images, it.N, it.H, it.W, it.level, it.Il, local * kTile); RL_PSB(-1); }
@@ -368,12 +365,12 @@ k_select_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
 
 template <typename Tm, bool FROM_KEYS>
 void launch_select_t(const void* M, const float* keys, int D, int h, int w, int k, uint8_t* S, uint64_t* mask,
-                     uint8_t* slots, float* Gzero, unsigned* counter_zero, int mode, cudaStream_t s) {
+                     uint8_t* slots, float* Gzero, int mode, cudaStream_t s) {
     const long long hw = (long long)h * w;
     const int blocks = (int)((hw + 127) / 128);
 #define RL_SEL(KK)                                                                                          \
     k_select<Tm, FROM_KEYS, KK><<<blocks, 128, 0, s>>>((const Tm*)M, keys, D, h, w, k, S, mask, slots, Gzero, \
-                                                       counter_zero, mode)
+                                                       mode)
     switch (mode == 1 ? 1 : k) {
         case 1: RL_SEL(1); break;
         case 2: RL_SEL(2); break;
@@ -390,12 +387,12 @@ void launch_select_t(const void* M, const float* keys, int D, int h, int w, int 
 
 template <typename Tm, int LOG>
 void launch_pyramid_select_l(const Tm* M, int D, int H, int W, int level, Tm* Ml, int k, uint8_t* S,
-                             uint8_t* slots, float* Gzero, unsigned* counter_zero, int mode, cudaStream_t s,
+                             uint8_t* slots, float* Gzero, int mode, cudaStream_t s,
                              const float* images, int N, float* Il) {
     const long long hw = (long long)(H >> level) * (W >> level);
     const unsigned blocks = (unsigned)((hw + kTile - 1) / kTile);
 #define RL_PS(KK)                                                                                                 \
-    k_pyramid_select<Tm, KK, LOG><<<blocks, 256, 0, s>>>(M, D, H, W, level, Ml, k, S, slots, Gzero, counter_zero, mode, \
+    k_pyramid_select<Tm, KK, LOG><<<blocks, 256, 0, s>>>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, \
                                                          images, N, Il)
     switch (mode == 1 ? 1 : k) {
         case 1: RL_PS(1); break;
@@ -413,17 +410,14 @@ void launch_pyramid_select_l(const Tm* M, int D, int H, int W, int level, Tm* Ml
 
 template <typename Tm>
 void launch_pyramid_select_t(const void* M, int D, int H, int W, int level, void* Ml, int k, uint8_t* S,
-                             uint8_t* slots, float* Gzero, unsigned* counter_zero, int mode, cudaStream_t s,
+                             uint8_t* slots, float* Gzero, int mode, cudaStream_t s,
                              const float* images, int N, float* Il) {
     if (level == 1)
-        launch_pyramid_select_l<Tm, 1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, counter_zero,
-                                       mode, s, images, N, Il);
+        launch_pyramid_select_l<Tm, 1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il);
     else if (level == 2)
-        launch_pyramid_select_l<Tm, 2>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, counter_zero,
-                                       mode, s, images, N, Il);
+        launch_pyramid_select_l<Tm, 2>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il);
     else
-        launch_pyramid_select_l<Tm, -1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, counter_zero,
-                                        mode, s, images, N, Il);
+        launch_pyramid_select_l<Tm, -1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il);
 }
 
 __global__ void k_mask_to_slots(const uint64_t* __restrict__ mask, int D, int k, int hw,
@@ -460,32 +454,31 @@ __global__ void k_downsample_f32(const float* __restrict__ x, int P, int H, int 
 }  // namespace
 
 rl_status rl_launch_select(const void* M, rl_dtype dt, const float* keys, int D, int h, int w, int k, uint8_t* S,
-                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, unsigned* counter_zero,
-                           int mode) {
+                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, int mode) {
     if (keys) {
         RLTraceScope ts("select_keys", s);
-        launch_select_t<float, true>(nullptr, keys, D, h, w, k, S, mask, slots, Gzero, counter_zero, mode, s);
+        launch_select_t<float, true>(nullptr, keys, D, h, w, k, S, mask, slots, Gzero, mode, s);
     } else if (dt == RL_F32) {
         RLTraceScope ts("select_f32", s);
-        launch_select_t<float, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, counter_zero, mode, s);
+        launch_select_t<float, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, mode, s);
     } else {
         RLTraceScope ts("select_bf16", s);
-        launch_select_t<__nv_bfloat16, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, counter_zero, mode, s);
+        launch_select_t<__nv_bfloat16, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, mode, s);
     }
     return rl_check_launch("select");
 }
 
 rl_status rl_launch_pyramid_select(const void* M, rl_dtype dt, int D, int H, int W, int level, void* Ml, int k,
-                                   uint8_t* S, uint8_t* slots, float* Gzero, unsigned* counter_zero, int mode,
+                                   uint8_t* S, uint8_t* slots, float* Gzero, int mode,
                                    cudaStream_t s, const float* images, int N, float* Il) {
     if (!images) Il = nullptr;
     if (dt == RL_F32) {
         RLTraceScope ts("pyramid_select_f32", s);
-        launch_pyramid_select_t<float>(M, D, H, W, level, Ml, k, S, slots, Gzero, counter_zero, mode, s, images, N,
+        launch_pyramid_select_t<float>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, s, images, N,
                                        Il);
     } else {
         RLTraceScope ts("pyramid_select_bf16", s);
-        launch_pyramid_select_t<__nv_bfloat16>(M, D, H, W, level, Ml, k, S, slots, Gzero, counter_zero, mode, s,
+        launch_pyramid_select_t<__nv_bfloat16>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, s,
                                                images, N, Il);
     }
     return rl_check_launch("pyramid_select");

@@ -40,6 +40,18 @@ int rl_kernel_path(int H, int W, int nviews) {
     return (long long)H * W * nviews < (1ll << 19) ? 3 : 2;
 }
 
+int rl_grad_path(int H, int W, int nviews, bool anchored) {
+    const int p = g_path.load(std::memory_order_relaxed);
+    if (p != 0) return p >= 3 ? 3 : p;
+    return anchored && (long long)H * W * nviews >= (1ll << 19) ? 2 : 3;
+}
+
+int rl_batch_grad_path(long long pixel_views) {
+    const int p = g_path.load(std::memory_order_relaxed);
+    if (p != 0) return p >= 3 ? 3 : p;
+    return pixel_views < (1ll << 19) ? 3 : 2;
+}
+
 unsigned int* rl_device_status_ptr() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return nullptr;

@@ -7,6 +7,11 @@
 // Only k of the D planes are read and written.  With lambda_s != 0 the sparsity prior of
 // Sec. 3.4 joins the alpha step: lambda_s sign(0.5 - a) / ((1.5 - |0.5 - a|) h w D), with a
 // the alpha of the level MPI Ml.
+//
+// The launch also sums the gradient's loss partials, in one block of its own beside the update's
+// (512x384: no measurable time).  Summing them at the end of the gradient instead made every one of
+// its blocks fence its reductions and wait for them: 272 against 233 us at level 0 of 512x384,
+// D = 32, 4 views, FP32.
 #include <type_traits>
 
 #include "rl_internal.h"
@@ -52,13 +57,22 @@ __device__ __forceinline__ void update_pixel(Tm* __restrict__ M, int D, int H, i
 template <typename Tm>
 __global__ void __launch_bounds__(128)
 k_update(Tm* __restrict__ M, int D, int H, int W, int level, const uint8_t* __restrict__ S,
-         const float* __restrict__ G, int k, float lambda, int clamp01, const Tm* __restrict__ Ml, float prior_scale) {
+         const float* __restrict__ G, int k, float lambda, int clamp01, const Tm* __restrict__ Ml, float prior_scale,
+         const RLLossSum loss) {
+    if (blockIdx.y == (unsigned)H) {  // a row of its own: the sum overlaps the update's blocks
+        if (blockIdx.x != 0) return;
+        __shared__ float red[4];
+        const float total = rl_partials_sum(loss.partials, (unsigned)loss.n, threadIdx.x, 128, red);
+        if (threadIdx.x == 0) loss.out[0] = total * loss.scale;
+        return;
+    }
     update_pixel<Tm>(M, D, H, W, level, S, G, k, lambda, clamp01, Ml, prior_scale, blockIdx.x * blockDim.x + threadIdx.x,
                      blockIdx.y);
 }
 
 // Batched update: one persistent launch walks the update units of every item of a batch table
-// (a unit is 128 pixels of one full-resolution row of one item, as k_update's grid).
+// (a unit is 128 pixels of one full-resolution row of one item, as k_update's grid; an item's
+// last unit sums its loss).
 template <typename Tm>
 __global__ void __launch_bounds__(128)
 k_update_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restrict__ items) {
@@ -68,6 +82,13 @@ k_update_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
     for (unsigned u = rl_batch_next(hdr, 3, &next_slot); u < total; u = rl_batch_next(hdr, 3, &next_slot)) {
         const RLBatchItem& it = items[rl_batch_find(items, n, u, &RLBatchItem::upd_begin)];
         const unsigned local = u - it.upd_begin;
+        if (local == it.upd_units - 1) {  // the item's last unit: its loss
+            if (!it.loss_out) continue;
+            __shared__ float red[4];
+            const float total = rl_partials_sum(it.partials, it.parts, threadIdx.x, 128, red);
+            if (threadIdx.x == 0) it.loss_out[0] = total * it.loss_scale;
+            continue;
+        }
         const int x = (int)(local % it.upd_tiles_x) * 128 + threadIdx.x, y = (int)(local / it.upd_tiles_x);
         update_pixel<Tm>(static_cast<Tm*>(it.M), it.D, it.H, it.W, it.level, it.S, it.G, it.k, it.lambda, it.clamp01,
                          static_cast<const Tm*>(it.Ml), it.prior_scale, x, y);
@@ -77,19 +98,19 @@ k_update_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
 }  // namespace
 
 rl_status rl_launch_update(void* M, rl_dtype dt, int D, int H, int W, int level, const uint8_t* S, const float* G,
-                           int k, float lambda, int clamp01, cudaStream_t s, const void* Ml, float lambda_s) {
-    dim3 grid((W + 127) / 128, H);
+                           int k, float lambda, int clamp01, cudaStream_t s, const void* Ml, float lambda_s, const RLLossSum& loss) {
+    dim3 grid((W + 127) / 128, H + (loss.out ? 1 : 0));
     // lambda_s / (h w D): the mean in L_s is over the level MPI's voxels
     const float prior_scale =
         (Ml && lambda_s != 0.f) ? (float)((double)lambda_s / ((double)(H >> level) * (W >> level) * D)) : 0.f;
     if (dt == RL_F32) {
         RLTraceScope ts("update_f32", s);
         k_update<float><<<grid, 128, 0, s>>>((float*)M, D, H, W, level, S, G, k, lambda, clamp01, (const float*)Ml,
-                                             prior_scale);
+                                             prior_scale, loss);
     } else {
         RLTraceScope ts("update_bf16", s);
         k_update<__nv_bfloat16><<<grid, 128, 0, s>>>((__nv_bfloat16*)M, D, H, W, level, S, G, k, lambda, clamp01,
-                                                     (const __nv_bfloat16*)Ml, prior_scale);
+                                                     (const __nv_bfloat16*)Ml, prior_scale, loss);
     }
     return rl_check_launch("update");
 }

@@ -20,7 +20,7 @@
 // the latency of the gathers.  Both passes take the planes in groups of two, whose loads are in
 // flight together, and pass 2 forms the T_d within a group from the group's stored one: half the
 // shared memory, so that a launch of 64 planes keeps 32 warps an SM instead of 24 and its L1.
-// 1920x1080, D = 64, 8 views, BF16, anchored: 9.03 ms (one plane at a time 11.56 ms, groups of four
+// 1920x1080, D = 64, 8 views, BF16, anchored: 8.53 ms (one plane at a time 11.56 ms, groups of four
 // 10.8 ms; at the start, with border tests in every sample and a fenced loss reduction at the end
 // of every block, 12.9 ms).
 #include <type_traits>
@@ -46,7 +46,7 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
     __shared__ RLAnchor sA;  // the tile's anchor: its centre pixel
     if (ANCH)
         rl_anchor_build(&sA, views, view, (qx & ~(kGradBX - 1)) + kGradBX / 2, qy - qy % kGradBY + kGradBY / 2, D,
-                        tid, kGradThreads);
+                        W, tid, kGradThreads);
     const unsigned act = __ballot_sync(0xffffffffu, qx < W && qy < H);
     if (qx < W && qy < H) {
         const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[view], qx, qy);
@@ -68,14 +68,14 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
 #pragma unroll
                 for (int i = kGroup - 1; i >= 0; --i) {
                     const int d = min(j * kGroup + i, D - 1);
-                    m[i] = inside(d, rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W));
+                    m[i] = inside(d, rl_fast_tap<ANCH>(w, sA, views, d, base, W));
                     if (j * kGroup + i >= D) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             } else {
 #pragma unroll
                 for (int i = kGroup - 1; i >= 0; --i) {
                     const int d = j * kGroup + i;
-                    m[i] = d < D ? rl_sample(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
+                    m[i] = d < D ? rl_sample_fast(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
                                  : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
@@ -128,7 +128,7 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
 #pragma unroll
                 for (int i = kGroup - 1; i >= 0; --i) {
                     const int d = min(j * kGroup + i, D - 1);
-                    const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                    const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
                     m[i] = inside(d, t);
                     if (SPARSE) word[i] = rl_slot_word(slots, (unsigned)d * hw + t.idx, W);
                     if (j * kGroup + i >= D) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -138,7 +138,7 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
                 for (int i = kGroup - 1; i >= 0; --i) {
                     const int d = j * kGroup + i;
                     word[i] = 0u;
-                    m[i] = d < D ? rl_sample(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
+                    m[i] = d < D ? rl_sample_fast(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
                                  : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
@@ -156,7 +156,7 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
                     const float4 g = make_float4(gc * r0, gc * r1, gc * r2,
                                                  Td[i] * fmaf(m[i].x - b0, r0, fmaf(m[i].y - b1, r1, (m[i].z - b2) * r2)));
                     if (fast) {
-                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
                         rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W, t.fx,
                                               t.fy, g, ng);
                     } else {

@@ -76,7 +76,7 @@ k_render_pp(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant
     __shared__ RLAnchor sA;
     const PixelCoord pc = pixel_coord(H, W);
     if (ANCH)
-        rl_anchor_build(&sA, views, pc.view, blockIdx.y * kTX + kTX / 2, blockIdx.z * kTY + kTY / 2, D, threadIdx.x,
+        rl_anchor_build(&sA, views, pc.view, blockIdx.y * kTX + kTX / 2, blockIdx.z * kTY + kTY / 2, D, W, threadIdx.x,
                         kGroups * kPix);
     const int qx = min(pc.qx, W - 1), qy = min(pc.qy, H - 1);
     const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[pc.view], qx, qy);
@@ -184,7 +184,7 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
     __shared__ RLAnchor sA;
     if (ANCH)
         rl_anchor_build(&sA, views, pc.view, bx * sh.tiles * sh.tile_x + sh.tiles * sh.tile_x / 2,
-                        pc.ty * (kPix / sh.tile_x), D, threadIdx.x, blockDim.x);
+                        pc.ty * (kPix / sh.tile_x), D, W, threadIdx.x, blockDim.x);
     const int qx = min(pc.qx, W - 1), qy = min(pc.qy, H - 1);
     const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[pc.view], qx, qy);
     const unsigned hw = (unsigned)(H * W);
@@ -213,7 +213,7 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
 #pragma unroll
         for (int i = C - 1; i >= 0; --i) {
             const int d = FULL ? d0 + i : d0 + min(i, n - 1);
-            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
             m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             word[i] = 0xFFFFFFFFu;
             if (RL_IN((long long)t.idx + W + 1, hw)) {
@@ -321,7 +321,7 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
                     g.z = gc * r2;
                     g.w = Td * fmaf(mi.x - b0, r0, fmaf(mi.y - b1, r1, (mi.z - b2) * r2));
                     if (fast) {  // the taps are formed again: keeping them costs registers, and warps
-                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
                         rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W, t.fx,
                                               t.fy, g, ng);
                     } else {

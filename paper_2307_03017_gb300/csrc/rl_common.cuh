@@ -224,15 +224,24 @@ struct RLPlaneK {
 };
 #define RL_PLANE_NONE (-0x40000000)
 
+// What a sample known to lie inside the plane needs of plane d, in one 16-byte load: the fraction,
+// the integer part as a voxel offset iy W + ix, and the plane's inverse depth.
+struct RLPlaneF {
+    float fx, fy;
+    int off;
+    float rho;
+};
+
 struct RLAnchor {
     float mx, my, ez, Nx, Ny, Dc;  // anchor quantities (FP32) for the per-pixel differences
     int u, v;                      // anchor pixel
     RLPlaneK k[RL_DEV_MAX_PLANES];
+    RLPlaneF f[RL_DEV_MAX_PLANES];
 };
 
 // Fills A (shared memory) for view `view` of V at anchor pixel (u, v).  Every thread of the
-// block calls it (it synchronises the block twice); nthreads threads, index tid.
-__device__ __forceinline__ void rl_anchor_build(RLAnchor* A, const RLViews& V, int view, int u, int v, int D,
+// block calls it (it synchronises the block twice); nthreads threads, index tid; W the plane's width.
+__device__ __forceinline__ void rl_anchor_build(RLAnchor* A, const RLViews& V, int view, int u, int v, int D, int W,
                                                 int tid, int nthreads) {
     __shared__ double s_ab[4];
     const RLViewParam64& P = V.v64[view];
@@ -278,6 +287,7 @@ __device__ __forceinline__ void rl_anchor_build(RLAnchor* A, const RLViews& V, i
             k.fx = k.fy = 0.f;
         }
         A->k[d] = k;
+        A->f[d] = RLPlaneF{k.fx, k.fy, (int)((unsigned)k.iy * (unsigned)W + (unsigned)k.ix), V.rho[d]};
     }
     __syncthreads();
 }
@@ -526,15 +536,16 @@ __device__ __forceinline__ unsigned rl_fast_base(int qx, int qy, int W) {
 }
 
 template <bool ANCH>
-__device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const RLAnchor& A, int d, float rho,
-                                            unsigned base, int W) {
+__device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const RLAnchor& A, const RLViews& views,
+                                                 int d, unsigned base, int W) {
     float sx, sy;
     if constexpr (ANCH) {
-        const RLPlaneK k = A.k[d];
-        sx = k.fx + fmaf(rho, w.w.dbx, w.w.dax);
-        sy = k.fy + fmaf(rho, w.w.dby, w.w.day);
-        base += (unsigned)(k.iy * W + k.ix);
+        const RLPlaneF k = A.f[d];
+        sx = k.fx + fmaf(k.rho, w.w.dbx, w.w.dax);
+        sy = k.fy + fmaf(k.rho, w.w.dby, w.w.day);
+        base += (unsigned)k.off;
     } else {
+        const float rho = views.rho[d];
         sx = fmaf(rho, w.w.bx, w.w.ax);
         sy = fmaf(rho, w.w.by, w.w.ay);
     }
@@ -680,13 +691,20 @@ __device__ __forceinline__ float rl_partials_sum(const float* __restrict__ parti
                                                  float* red) {
     float a[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
     const unsigned n4 = n / 4;
-#pragma unroll 8
-    for (unsigned i = tid; i < n4; i += nthreads) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(partials) + i);
-        rl_kahan_add(a[0], c[0], v.x);
-        rl_kahan_add(a[1], c[1], v.y);
-        rl_kahan_add(a[2], c[2], v.z);
-        rl_kahan_add(a[3], c[3], v.w);
+    for (unsigned i = tid; i < n4; i += 8 * nthreads) {
+        float4 v[8];  // eight loads in flight: one block reads them all
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const unsigned e = i + u * nthreads;
+            v[u] = e < n4 ? __ldcg(reinterpret_cast<const float4*>(partials) + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            rl_kahan_add(a[0], c[0], v[u].x);
+            rl_kahan_add(a[1], c[1], v[u].y);
+            rl_kahan_add(a[2], c[2], v[u].z);
+            rl_kahan_add(a[3], c[3], v[u].w);
+        }
     }
     if (tid < (int)(n & 3u)) rl_kahan_add(a[0], c[0], __ldcg(partials + n4 * 4 + tid));
     const float acc = rl_warp_sum((a[0] + a[1]) + (a[2] + a[3]));

@@ -67,7 +67,7 @@ k_view_alpha(const Tm* __restrict__ M, int D, int H, int W, const __grid_constan
     const int view = blockIdx.x;  // grid (views, tiles_x, tiles_y)
     if (ANCH)
         rl_anchor_build(&sA, views, view, blockIdx.y * kAlphaBX + kAlphaBX / 2, blockIdx.z * kAlphaBY + kAlphaBY / 2,
-                        D, threadIdx.y * kAlphaBX + threadIdx.x, kAlphaBX * kAlphaBY);
+                        D, W, threadIdx.y * kAlphaBX + threadIdx.x, kAlphaBX * kAlphaBY);
     const int qx = blockIdx.y * kAlphaBX + threadIdx.x;
     const int qy = blockIdx.z * kAlphaBY + threadIdx.y;
     if (qx >= W || qy >= H) return;

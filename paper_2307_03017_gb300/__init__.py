@@ -11,6 +11,7 @@ device.
 from __future__ import annotations
 
 import ctypes
+import struct
 
 import numpy as np
 import torch
@@ -33,6 +34,7 @@ RealLifeError = _lib.RealLifeError
 F32, BF16 = 0, 1
 SELECT_TOPK, SELECT_MVS = 0, 1
 _DT = {torch.float32: F32, torch.bfloat16: BF16}
+_MPI_HEAD = struct.Struct("@iiiddiP")  # the fields of rl_mpi before its camera, in C alignment
 
 
 def library_path() -> str:
@@ -67,13 +69,10 @@ class Mpi:
         return self.data.shape[2]
 
     def c_struct(self) -> _lib.RlMpi:
-        s = _lib.RlMpi()
-        s.D, s.H, s.W = self.D, self.H, self.W
-        s.near_, s.far_ = self.near, self.far
-        s.dtype = _DT[self.data.dtype]
-        s.data = ctypes.c_void_p(self.data.data_ptr())
-        s.ref = _lib.camera(self.ref)
-        return s
+        d = self.data
+        D, H, W, _ = d.shape
+        return _lib.RlMpi.from_buffer_copy(
+            _MPI_HEAD.pack(D, H, W, self.near, self.far, _DT[d.dtype], d.data_ptr()) + _lib.camera_bytes(self.ref))
 
 
 def make_mpi(data: torch.Tensor, near: float, far: float, ref) -> Mpi:
@@ -82,7 +81,8 @@ def make_mpi(data: torch.Tensor, near: float, far: float, ref) -> Mpi:
 
 def _stream(stream) -> ctypes.c_void_p:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        # the current device's current stream, without the Stream object around it (3 us)
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 

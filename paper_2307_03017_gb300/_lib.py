@@ -66,21 +66,26 @@ class RlTraceEntry(ctypes.Structure):
     _fields_ = [("name", ctypes.c_char * 48), ("launches", ctypes.c_longlong), ("total_ms", ctypes.c_double)]
 
 
-def camera(c) -> RlCamera:
-    """Host camera struct from an object with K, R, t (or a (K, R, t) tuple)."""
+def _f64(a, n: int) -> bytes:
+    """The n values of `a`, row-major, as float64 bytes."""
+    a = np.asarray(a, dtype=np.float64)
+    return (a if a.size == n else a.reshape(n)).tobytes()
+
+
+def camera_bytes(c) -> bytes:
+    """The camera struct's bytes (its fields are 21 doubles) from an object with K, R, t (or a
+    (K, R, t) tuple).  One copy a field: filling a ctypes array value by value takes longer than
+    launching a small render (2.3 us a camera, against 1.1 us)."""
     K, R, t = (c.K, c.R, c.t) if hasattr(c, "K") else c
-    s = RlCamera()
-    s.K[:] = np.asarray(K, dtype=np.float64).reshape(9).tolist()
-    s.R[:] = np.asarray(R, dtype=np.float64).reshape(9).tolist()
-    s.t[:] = np.asarray(t, dtype=np.float64).reshape(3).tolist()
-    return s
+    return _f64(K, 9) + _f64(R, 9) + _f64(t, 3)
+
+
+def camera(c) -> RlCamera:
+    return RlCamera.from_buffer_copy(camera_bytes(c))
 
 
 def cameras(cs):
-    arr = (RlCamera * len(cs))()
-    for i, c in enumerate(cs):
-        arr[i] = camera(c)
-    return arr
+    return (RlCamera * len(cs)).from_buffer_copy(b"".join([camera_bytes(c) for c in cs]))
 
 
 def path() -> str:

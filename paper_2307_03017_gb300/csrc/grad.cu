@@ -2,8 +2,8 @@
 // all source views), the render backward used by autograd, and the loss reduction.
 //
 // Per view pixel q (one thread), with T_d = prod_{j>d}(1 - alpha_j) (Eq. eq_over):
-//   pass 1, d = D-1 .. 0:  m_d = bilinear(M[d], p_d(q)); T_d of every kGroup-th plane -> shared
-//                           memory; C += T_d alpha_d c_d; T *= (1 - alpha_d)
+//   pass 1, d = D-1 .. 0:  m_d = bilinear(M[d], p_d(q)); T_d of each group's nearest plane ->
+//                           shared memory; C += T_d alpha_d c_d; T *= (1 - alpha_d)
 //   residual:               r = (C - I(q)) / N  (loss mode; L = 1/(2N) sum |C - I|^2; I the
 //                           level image: given at the level's resolution, img_level 0, or formed
 //                           on the fly from its 2^l x 2^l full-resolution pixels)
@@ -17,12 +17,12 @@
 // the pixel) or RL_SLOT_NONE.  No division by (1 - alpha).
 //
 // What bounds it: L1 wavefronts (two gathers a sample and the reductions onto the kept taps) and
-// the latency of the gathers.  Both passes take the planes in groups of two, whose loads are in
-// flight together, and pass 2 forms the T_d within a group from the group's stored one: half the
-// shared memory, so that a launch of 64 planes keeps 32 warps an SM instead of 24 and its L1.
-// 1920x1080, D = 64, 8 views, BF16, anchored: 8.53 ms (one plane at a time 11.56 ms, groups of four
-// 10.8 ms; at the start, with border tests in every sample and a fenced loss reduction at the end
-// of every block, 12.9 ms).
+// the latency of the gathers.  Warps whose samples all lie inside leave out the border tests.  With
+// many planes both passes take them in pairs, whose loads are in flight together, and pass 2 forms
+// T_d within a pair from the pair's stored one: half the shared memory, so that a launch of 64
+// planes keeps 32 warps an SM instead of 24, and its L1.  1920x1080, D = 64, 8 views, BF16, anchored:
+// 8.23 ms (one plane at a time 11.56 ms, groups of four 10.8 ms; at the start, with border tests in
+// every sample and a fenced loss reduction at the end of every block, 12.9 ms).
 #include <type_traits>
 
 #include "rl_internal.h"
@@ -30,12 +30,12 @@
 namespace {
 
 constexpr int kGradBX = 32, kGradBY = 4, kGradThreads = kGradBX * kGradBY;
-constexpr int kGroup = 2;           // planes whose samples are held together
-constexpr int kGradMinBlocks = 8;   // resident blocks the registers must allow (10: 9.28 ms, 6: 10.5 ms)
+constexpr int kGroup = 2;          // planes whose samples are held together (grad_group, the batch)
+constexpr int kGradMinBlocks = 8;  // resident blocks the registers must then allow
 
 // One block's tile of 32 x 4 view pixels of one view.  bid / nblocks index the block among
 // the launch's (or the batch item's) blocks for the loss partials.
-template <typename Tm, bool SPARSE, bool LOSS, bool ANCH>
+template <typename Tm, int GROUP, bool SPARSE, bool LOSS, bool ANCH>
 __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H, int W, const RLViews& views, int view,
                                           int qx, int qy, int tid, float* __restrict__ sT,
                                           const float* __restrict__ images, int img_level,
@@ -54,41 +54,39 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
         const unsigned hw = (unsigned)(H * W), base = rl_fast_base(qx, qy, W);
         // warps whose samples of every plane lie inside it skip the border tests
         const bool fast = __all_sync(act, rl_chunk_inside<ANCH>(w, sA, views, 0, D - 1, qx, qy, H, W));
-        // the sample of plane d (transparent beyond the last plane)
-        const auto inside = [&](int d, const RLFastTap& t) {
-            return RL_IN((long long)t.idx + W + 1, hw) ? rl_sample_at(M, (unsigned)d * hw + t.idx, W, t.fx, t.fy)
-                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-        };
-        const int groups = (D + kGroup - 1) / kGroup;
+        const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int groups = (D + GROUP - 1) / GROUP;
         float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
+        // the two kinds of warp take separate loops: a branch in every group costs 15%
+        const auto pass1 = [&](auto inside) {
 #pragma unroll 1
-        for (int j = groups - 1; j >= 0; --j) {
-            float4 m[kGroup];
-            if (fast) {
+            for (int j = groups - 1; j >= 0; --j) {
+                float4 m[GROUP];
 #pragma unroll
-                for (int i = kGroup - 1; i >= 0; --i) {
-                    const int d = min(j * kGroup + i, D - 1);
-                    m[i] = inside(d, rl_fast_tap<ANCH>(w, sA, views, d, base, W));
-                    if (j * kGroup + i >= D) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = GROUP - 1; i >= 0; --i) {
+                    const int d = j * GROUP + i, dc = GROUP == 1 ? d : min(d, D - 1);
+                    if constexpr (decltype(inside)::value) {
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, dc, base, W);
+                        m[i] = RL_IN((long long)t.idx + W + 1, hw)
+                                   ? rl_sample_at(M, (unsigned)dc * hw + t.idx, W, t.fx, t.fy) : none;
+                    } else {
+                        m[i] = rl_sample_fast(M + dc * plane, H, W, w.taps(sA, dc, views.rho[dc], qx, qy));
+                    }
+                    if (GROUP > 1 && d >= D) m[i] = none;  // beyond the last plane
                 }
-            } else {
+                sT[j * kGradThreads + tid] = T;
 #pragma unroll
-                for (int i = kGroup - 1; i >= 0; --i) {
-                    const int d = j * kGroup + i;
-                    m[i] = d < D ? rl_sample_fast(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int i = GROUP - 1; i >= 0; --i) {
+                    const float a = T * m[i].w;
+                    c0 = fmaf(a, m[i].x, c0);
+                    c1 = fmaf(a, m[i].y, c1);
+                    c2 = fmaf(a, m[i].z, c2);
+                    T = T * (1.f - m[i].w);
                 }
             }
-            sT[j * kGradThreads + tid] = T;
-#pragma unroll
-            for (int i = kGroup - 1; i >= 0; --i) {
-                const float a = T * m[i].w;
-                c0 = fmaf(a, m[i].x, c0);
-                c1 = fmaf(a, m[i].y, c1);
-                c2 = fmaf(a, m[i].z, c2);
-                T = T * (1.f - m[i].w);
-            }
-        }
+        };
+        if (fast) pass1(std::true_type());
+        else pass1(std::false_type());
         float r0, r1, r2;
         if (LOSS) {
             // source image at this level: mean of the 2^l x 2^l full-resolution block
@@ -119,57 +117,63 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
         }
         float b0 = 0.f, b1 = 0.f, b2 = 0.f;
         const unsigned ng = views.gplanes ? (unsigned)views.gplanes : (unsigned)D;  // checked in debug builds
+        const auto pass2 = [&](auto inside) {
 #pragma unroll 1
-        for (int j = 0; j < groups; ++j) {
-            float4 m[kGroup];
-            float Td[kGroup];
-            unsigned word[kGroup];
-            if (fast) {
+            for (int j = 0; j < groups; ++j) {
+                float4 m[GROUP];
+                float Td[GROUP];
+                unsigned word[GROUP];
+                RLFastTap tap[GROUP];
 #pragma unroll
-                for (int i = kGroup - 1; i >= 0; --i) {
-                    const int d = min(j * kGroup + i, D - 1);
-                    const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
-                    m[i] = inside(d, t);
-                    if (SPARSE) word[i] = rl_slot_word(slots, (unsigned)d * hw + t.idx, W);
-                    if (j * kGroup + i >= D) m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            } else {
-#pragma unroll
-                for (int i = kGroup - 1; i >= 0; --i) {
-                    const int d = j * kGroup + i;
-                    word[i] = 0u;
-                    m[i] = d < D ? rl_sample_fast(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy))
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-            }
-            float Tg = sT[j * kGradThreads + tid];
-#pragma unroll
-            for (int i = kGroup - 1; i >= 0; --i) {
-                Td[i] = Tg;
-                Tg = Tg * (1.f - m[i].w);
-            }
-#pragma unroll
-            for (int i = 0; i < kGroup; ++i) {
-                const int d = j * kGroup + i;
-                if (Td[i] != 0.f && d < D) {
-                    const float gc = Td[i] * m[i].w;
-                    const float4 g = make_float4(gc * r0, gc * r1, gc * r2,
-                                                 Td[i] * fmaf(m[i].x - b0, r0, fmaf(m[i].y - b1, r1, (m[i].z - b2) * r2)));
-                    if (fast) {
-                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
-                        rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W, t.fx,
-                                              t.fy, g, ng);
+                for (int i = GROUP - 1; i >= 0; --i) {
+                    const int d = j * GROUP + i, dc = GROUP == 1 ? d : min(d, D - 1);
+                    if constexpr (decltype(inside)::value) {
+                        tap[i] = rl_fast_tap<ANCH>(w, sA, views, dc, base, W);
+                        const unsigned e = (unsigned)dc * hw + tap[i].idx;
+                        m[i] = none;
+                        word[i] = 0xFFFFFFFFu;
+                        if (RL_IN((long long)tap[i].idx + W + 1, hw)) {
+                            if (SPARSE) word[i] = rl_slot_word(slots, e, W);
+                            m[i] = rl_sample_at(M, e, W, tap[i].fx, tap[i].fy);
+                        }
                     } else {
-                        const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
-                        if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);
+                        m[i] = rl_sample_fast(M + dc * plane, H, W, w.taps(sA, dc, views.rho[dc], qx, qy));
                     }
+                    if (GROUP > 1 && d >= D) m[i] = none;
                 }
-                const float om = 1.f - m[i].w;
-                b0 = fmaf(m[i].x, m[i].w, om * b0);
-                b1 = fmaf(m[i].y, m[i].w, om * b1);
-                b2 = fmaf(m[i].z, m[i].w, om * b2);
+                float Tg = sT[j * kGradThreads + tid];
+#pragma unroll
+                for (int i = GROUP - 1; i >= 0; --i) {
+                    Td[i] = Tg;
+                    Tg = Tg * (1.f - m[i].w);
+                }
+#pragma unroll
+                for (int i = 0; i < GROUP; ++i) {
+                    const int d = j * GROUP + i;
+                    if (Td[i] != 0.f && d < D) {
+                        const float gc = Td[i] * m[i].w;
+                        const float4 g =
+                            make_float4(gc * r0, gc * r1, gc * r2,
+                                        Td[i] * fmaf(m[i].x - b0, r0, fmaf(m[i].y - b1, r1, (m[i].z - b2) * r2)));
+                        if constexpr (decltype(inside)::value) {
+                            // a pair forms its taps again (they cost registers); a single plane keeps them
+                            const RLFastTap t = GROUP == 1 ? tap[i] : rl_fast_tap<ANCH>(w, sA, views, d, base, W);
+                            rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W,
+                                                  t.fx, t.fy, g, ng);
+                        } else {
+                            const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
+                            if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);
+                        }
+                    }
+                    const float om = 1.f - m[i].w;
+                    b0 = fmaf(m[i].x, m[i].w, om * b0);
+                    b1 = fmaf(m[i].y, m[i].w, om * b1);
+                    b2 = fmaf(m[i].z, m[i].w, om * b2);
+                }
             }
-        }
+        };
+        if (fast) pass2(std::true_type());
+        else pass2(std::false_type());
     }
     if (LOSS) {
         __shared__ float red[kGradThreads / 32];
@@ -184,14 +188,14 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
     }
 }
 
-template <typename Tm, bool SPARSE, bool LOSS, bool ANCH>
-__global__ void __launch_bounds__(kGradThreads, kGradMinBlocks)
+template <typename Tm, int GROUP, bool SPARSE, bool LOSS, bool ANCH>
+__global__ void __launch_bounds__(kGradThreads, GROUP == 1 ? 10 : kGradMinBlocks)
 k_grad(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views,
        const float* __restrict__ images, int img_level, const float* __restrict__ grad_out,
        const uint8_t* __restrict__ slots, float* __restrict__ G, float inv_n, float* __restrict__ partials) {
-    extern __shared__ float sT[];  // [ceil(D / kGroup)][kGradThreads]
+    extern __shared__ float sT[];  // [ceil(D / GROUP)][kGradThreads]
     // view-fastest block order: the N views of a tile run together and share M through L2
-    grad_tile<Tm, SPARSE, LOSS, ANCH>(M, D, H, W, views, blockIdx.x, blockIdx.y * kGradBX + threadIdx.x,
+    grad_tile<Tm, GROUP, SPARSE, LOSS, ANCH>(M, D, H, W, views, blockIdx.x, blockIdx.y * kGradBX + threadIdx.x,
                                 blockIdx.z * kGradBY + threadIdx.y, threadIdx.y * kGradBX + threadIdx.x, sT, images,
                                 img_level, grad_out, slots, G, inv_n, partials,
                                 blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
@@ -220,7 +224,7 @@ k_grad_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restric
         const unsigned view = local % (unsigned)it.N, tile = local / (unsigned)it.N;
         const int tx = (int)(tile % it.grad_tiles_x), ty = (int)(tile / it.grad_tiles_x);
         const int h = it.H >> it.level, w = it.W >> it.level;
-#define RL_GB(A) grad_tile<Tm, true, true, A>(static_cast<const Tm*>(it.Ml), it.D, h, w, it.views, (int)view,    \
+#define RL_GB(A) grad_tile<Tm, kGroup, true, true, A>(static_cast<const Tm*>(it.Ml), it.D, h, w, it.views, (int)view,    \
                                              tx * kGradBX + threadIdx.x, ty * kGradBY + threadIdx.y, tid, sT,       \
                                              it.level ? it.Il : it.images, 0, nullptr, it.slots, it.G, it.inv_n,    \
                                              it.partials,                                                           \
@@ -240,12 +244,21 @@ __global__ void __launch_bounds__(1024) k_loss_reduce(const float* __restrict__ 
     if (threadIdx.x == 0) out[0] = total * scale;
 }
 
+// Planes a group: one (48 registers, 40 resident warps) while the stored transmittances, 512 bytes a
+// plane and block, leave room for the blocks and the L1, else two (64 registers, half the bytes).
+// Gradient of 1200x576, 4 anchored views, us, one against two: FP32 D = 32 723 / 757, D = 40 982 / 955,
+// D = 64 2204 / 1579; BF16 D = 32 653 / 713, D = 48 985 / 1037, D = 64 1633 / 1349.
+int grad_group(int D, bool f32) { return D <= (f32 ? 32 : 48) ? 1 : kGroup; }
+
 template <typename Tm, bool SPARSE, bool LOSS>
 void launch_grad_t(const void* M, int D, int H, int W, const RLViews& views, const float* images, int img_level,
                    const float* grad_out, const uint8_t* slots, float* G, float inv_n, float* partials,
-                   dim3 grid, size_t smem, cudaStream_t s) {
-    auto kern = views.anchored ? k_grad<Tm, SPARSE, LOSS, true> : k_grad<Tm, SPARSE, LOSS, false>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                   dim3 grid, cudaStream_t s) {
+    const int group = grad_group(D, sizeof(Tm) == 4);
+    const size_t smem = (size_t)((D + group - 1) / group) * kGradThreads * sizeof(float);
+    auto kern = group == 1
+                    ? (views.anchored ? k_grad<Tm, 1, SPARSE, LOSS, true> : k_grad<Tm, 1, SPARSE, LOSS, false>)
+                    : (views.anchored ? k_grad<Tm, kGroup, SPARSE, LOSS, true> : k_grad<Tm, kGroup, SPARSE, LOSS, false>);
     kern<<<grid, dim3(kGradBX, kGradBY), smem, s>>>((const Tm*)M, D, H, W, views, images, img_level, grad_out, slots, G,
                                                     inv_n, partials);
 }
@@ -261,20 +274,18 @@ size_t rl_grad_num_blocks(int H, int W, int N) {
 rl_status rl_launch_grad(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                          const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G,
                          float inv_n, float* partials, int* nblocks, cudaStream_t s) {
-    if (rl_grad_path(H, W, views.n, views.anchored != 0) != 2)
+    if (rl_grad_path(H, W, views.n, D, views.anchored != 0, slots != nullptr) != 2)
         return rl_launch_grad_pp(M, dt, D, H, W, views, mode_loss, images, img_level, grad_out, slots, G, inv_n,
                                  partials, nblocks, s);
     const int tiles_x = (W + kGradBX - 1) / kGradBX, tiles_y = (H + kGradBY - 1) / kGradBY;
     const dim3 grid((unsigned)views.n, (unsigned)tiles_x, (unsigned)tiles_y);
-    const size_t smem = (size_t)((D + kGroup - 1) / kGroup) * kGradThreads * sizeof(float);
     if (nblocks) *nblocks = (int)(grid.x * grid.y * grid.z);
     const bool sparse = slots != nullptr;
     const char* name = dt == RL_F32 ? (sparse ? "grad_sparse_f32" : "grad_dense_f32")
                                     : (sparse ? "grad_sparse_bf16" : "grad_dense_bf16");
     RLTraceScope ts(name, s);
 #define RL_GRAD_CASE(TM, SP, LS) \
-    launch_grad_t<TM, SP, LS>(M, D, H, W, views, images, img_level, grad_out, slots, G, inv_n, partials, grid, \
-                              smem, s)
+    launch_grad_t<TM, SP, LS>(M, D, H, W, views, images, img_level, grad_out, slots, G, inv_n, partials, grid, s)
     // a slot map comes with the loss mode only
 #define RL_KIND(TM)                                                                               \
     do {                                                                                          \

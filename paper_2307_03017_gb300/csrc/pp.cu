@@ -134,8 +134,9 @@ struct PPShape {
 };
 
 // Tile of the gradient over a W x H image: 32 x 1 pixels (512x384: 218 against 224 us with 16 x 2)
-// unless 16 x 2 needs fewer tiles (widths just above a multiple of 32).
+// unless 16 x 2 needs fewer tiles (widths just above a multiple of 32) or the grid is too high.
 __host__ __device__ inline int grad_pp_tile_x(int H, int W) {
+    if (H > 65535) return 16;
     return (W + 15) / 16 * ((H + 1) / 2) < (W + 31) / 32 * H ? 16 : 32;
 }
 

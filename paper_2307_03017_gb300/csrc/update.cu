@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(128)
 k_update(Tm* __restrict__ M, int D, int H, int W, int level, const uint8_t* __restrict__ S,
          const float* __restrict__ G, int k, float lambda, int clamp01, const Tm* __restrict__ Ml, float prior_scale,
          const RLLossSum loss) {
-    if (blockIdx.y == (unsigned)H) {  // a row of its own: the sum overlaps the update's blocks
+    if (loss.out && blockIdx.y == 0) {  // the first row of blocks: the sum overlaps the update's
         if (blockIdx.x != 0) return;
         __shared__ float red[4];
         const float total = rl_partials_sum(loss.partials, (unsigned)loss.n, threadIdx.x, 128, red);
@@ -67,12 +67,12 @@ k_update(Tm* __restrict__ M, int D, int H, int W, int level, const uint8_t* __re
         return;
     }
     update_pixel<Tm>(M, D, H, W, level, S, G, k, lambda, clamp01, Ml, prior_scale, blockIdx.x * blockDim.x + threadIdx.x,
-                     blockIdx.y);
+                     (int)blockIdx.y - (loss.out ? 1 : 0));
 }
 
 // Batched update: one persistent launch walks the update units of every item of a batch table
 // (a unit is 128 pixels of one full-resolution row of one item, as k_update's grid; an item's
-// last unit sums its loss).
+// first unit sums its loss).
 template <typename Tm>
 __global__ void __launch_bounds__(128)
 k_update_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restrict__ items) {
@@ -81,14 +81,14 @@ k_update_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
     __shared__ unsigned next_slot;
     for (unsigned u = rl_batch_next(hdr, 3, &next_slot); u < total; u = rl_batch_next(hdr, 3, &next_slot)) {
         const RLBatchItem& it = items[rl_batch_find(items, n, u, &RLBatchItem::upd_begin)];
-        const unsigned local = u - it.upd_begin;
-        if (local == it.upd_units - 1) {  // the item's last unit: its loss
+        if (u == it.upd_begin) {  // the item's first unit: its loss
             if (!it.loss_out) continue;
             __shared__ float red[4];
             const float total = rl_partials_sum(it.partials, it.parts, threadIdx.x, 128, red);
             if (threadIdx.x == 0) it.loss_out[0] = total * it.loss_scale;
             continue;
         }
+        const unsigned local = u - it.upd_begin - 1;
         const int x = (int)(local % it.upd_tiles_x) * 128 + threadIdx.x, y = (int)(local / it.upd_tiles_x);
         update_pixel<Tm>(static_cast<Tm*>(it.M), it.D, it.H, it.W, it.level, it.S, it.G, it.k, it.lambda, it.clamp01,
                          static_cast<const Tm*>(it.Ml), it.prior_scale, x, y);
@@ -98,7 +98,14 @@ k_update_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
 }  // namespace
 
 rl_status rl_launch_update(void* M, rl_dtype dt, int D, int H, int W, int level, const uint8_t* S, const float* G,
-                           int k, float lambda, int clamp01, cudaStream_t s, const void* Ml, float lambda_s, const RLLossSum& loss) {
+                           int k, float lambda, int clamp01, cudaStream_t s, const void* Ml, float lambda_s,
+                           const RLLossSum& loss_in) {
+    RLLossSum loss = loss_in;
+    if (loss.out && H >= 65535) {  // no row of blocks left for the loss
+        const rl_status st = rl_launch_loss_reduce(loss.partials, loss.n, loss.scale, loss.out, s);
+        if (st) return st;
+        loss.out = nullptr;
+    }
     dim3 grid((W + 127) / 128, H + (loss.out ? 1 : 0));
     // lambda_s / (h w D): the mean in L_s is over the level MPI's voxels
     const float prior_scale =

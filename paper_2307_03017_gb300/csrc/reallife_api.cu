@@ -575,6 +575,12 @@ rl_status rl_gradient_volume(const rl_mpi* m, const float* images, const rl_came
     void* Ml = level == 0 ? m->data : (void*)(base + L.Ml);
     uint8_t* S = S_out ? S_out : (uint8_t*)(base + L.S);
     float* A = (float*)(base + L.A);
+    // the level's alphas alone, for the view alpha weights: at level 0 in the place of the level MPI
+    // (unused there, and as large), above it behind the level's weights, which take at most a quarter
+    // of theirs; odd sizes have no room for them
+    void* alphas = nullptr;
+    if (level) alphas = base + L.A + align_up((size_t)N * m->D * h * w * sizeof(float));
+    else if (m->H % 2 == 0 && m->W % 2 == 0) alphas = base + L.Ml;
     RLViews views;
     st = make_views(m, src, N, level, views);
     if (st) return st;
@@ -588,11 +594,11 @@ rl_status rl_gradient_volume(const rl_mpi* m, const float* images, const rl_came
         iv.full[i] = inv_view_param(m->ref, src[i]);
     }
     st = level ? rl_launch_pyramid_select(m->data, m->dtype, m->D, m->H, m->W, level, Ml, k, S, nullptr, nullptr,
-                                          selection, stream)
+                                          selection, stream, nullptr, 0, nullptr, alphas)
                : rl_launch_select(Ml, m->dtype, nullptr, m->D, h, w, k, S, nullptr, nullptr, nullptr, stream,
-                                  selection);
+                                  selection, alphas);
     if (st) return st;
-    st = rl_launch_view_alpha(Ml, m->dtype, m->D, h, w, views, A, stream);
+    st = rl_launch_view_alpha(Ml, alphas, m->dtype, m->D, h, w, views, A, stream);
     if (st) return st;
     return rl_launch_volume(Ml, m->dtype, m->D, h, w, level, S, k, A, images, iv, V, stream, act);
 }

@@ -436,6 +436,7 @@ template <> struct RLStore<float> {
     static __device__ __forceinline__ float4 load4_nc(const float* p) { return *reinterpret_cast<const float4*>(p); }
     static __device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
     static __device__ __forceinline__ float load1(const float* p) { return __ldg(p); }
+    static __device__ __forceinline__ void store1(float* p, float v) { *p = v; }
     static __device__ __forceinline__ float round1(float v) { return v; }
 };
 
@@ -463,6 +464,7 @@ template <> struct RLStore<__nv_bfloat16> {
         *reinterpret_cast<uint2*>(p) = r;
     }
     static __device__ __forceinline__ float load1(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+    static __device__ __forceinline__ void store1(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
     // the value a store of v would hold
     static __device__ __forceinline__ float round1(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 };

@@ -95,17 +95,19 @@ rl_status rl_launch_render_pp(const void* M, rl_dtype dt, int D, int H, int W, c
 rl_status rl_launch_loss_reduce(const float* partials, int n, float scale, float* out, cudaStream_t s);
 
 // Top-k selection on the MPI M [D][h][w][4] (or on keys [D][h][w] when keys != NULL).
-// Outputs (each optional): S [k][h][w], mask [h][w], slot map [D][h][w]; Gzero
-// [k][h][w][4] is zeroed.
+// Outputs (each optional): S [k][h][w], mask [h][w], slot map [D][h][w], the MPI's alphas alone
+// [D][h][w] in its storage type; Gzero [k][h][w][4] is zeroed.
 rl_status rl_launch_select(const void* M, rl_dtype dt, const float* keys, int D, int h, int w, int k, uint8_t* S,
-                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, int mode = 0);
+                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, int mode = 0,
+                           void* alphas = nullptr);
 // Level-l MPI Ml [D][H>>l][W>>l][4] = Down^l(M) (level >= 1) and the selection on it in one pass: outputs as
 // rl_launch_select without the mask, identical values.  With images and Il != NULL it also writes the
 // level-l source images Il [N][H>>l][W>>l][3] (2^l x 2^l means of images [N][H][W][3], formed exactly as
 // the gradient kernels form them on the fly), which the gradient then reads at img_level 0.
 rl_status rl_launch_pyramid_select(const void* M, rl_dtype dt, int D, int H, int W, int level, void* Ml, int k,
                                    uint8_t* S, uint8_t* slots, float* Gzero, int mode, cudaStream_t s,
-                                   const float* images = nullptr, int N = 0, float* Il = nullptr);
+                                   const float* images = nullptr, int N = 0, float* Il = nullptr,
+                                   void* alphas = nullptr);
 // Slot map [D][h][w] from a selection mask [h][w]: the kept planes of a pixel in ascending order
 // take slots 0 .. k-1; kept planes beyond the first k get no slot.
 rl_status rl_launch_mask_to_slots(const uint64_t* mask, int D, int k, int hw, uint8_t* slots, cudaStream_t s);
@@ -166,8 +168,9 @@ rl_status rl_launch_image_metrics(const float* x, const float* y, int N, int H, 
 rl_status rl_launch_kept_mass(const void* M, rl_dtype dt, int D, int H, int W, const uint64_t* mask, double* out,
                               double* partials, cudaStream_t s);
 
-// Alpha weights of the MPI warped into each view (Eq. eq_gradient): A device [N][D][H][W].
-rl_status rl_launch_view_alpha(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, float* A,
+// Alpha weights of the MPI warped into each view (Eq. eq_gradient): A device [N][D][H][W], from
+// the alphas alone [D][H][W] when given, else from the MPI's.
+rl_status rl_launch_view_alpha(const void* M, const void* alphas, rl_dtype dt, int D, int H, int W, const RLViews& views, float* A,
                                cudaStream_t s);
 // Sparsified gradient volume V [4N+4][k][h][w] from the level MPI Ml [D][h][w][4], the
 // selection S [k][h][w], the view alpha weights A [N][D][h][w] and full-resolution images.

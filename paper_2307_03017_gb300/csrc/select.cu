@@ -29,7 +29,8 @@ namespace {
 __device__ __forceinline__ bool beats(float a, int ia, float b, int ib) { return a > b || (a == b && ia < ib); }
 
 // Per-pixel selection.  raw_at(d) gives alpha_d (keys mode: the key of plane d).  Returns the
-// 64-bit mask of the kept planes.
+// 64-bit mask of the kept planes.  store_at(d, raw) sees every value once its batch has been loaded
+// (a store between the loads would hold them up).
 //   K <= 8: a register-resident list of the K best, sorted by (key descending, d ascending);
 //   its first k <= K entries are kept.  The walk
 //   visits the planes in descending d, so a new plane is below every listed one and wins
@@ -37,8 +38,13 @@ __device__ __forceinline__ bool beats(float a, int ia, float b, int ib) { return
 //   `>=` compare-exchanges.  Planes that cannot enter cost one comparison.
 //   K == 64: rank counting over the D keys (O(D^2), kept in local memory).
 // mode 1 (MVS sampling) keeps the k consecutive planes around the argmax of the keys.
-template <int K, bool FROM_KEYS, typename RawFn>
-__device__ __forceinline__ uint64_t select_mask(const RawFn& raw_at, int D, int k, int mode) {
+struct NoStore {
+    __device__ __forceinline__ void operator()(int, float) const {}
+};
+
+template <int K, bool FROM_KEYS, typename RawFn, typename StoreFn = NoStore>
+__device__ __forceinline__ uint64_t select_mask(const RawFn& raw_at, int D, int k, int mode,
+                                                const StoreFn& store_at = StoreFn()) {
     constexpr bool SMALL = K <= 8;
     float kv[SMALL ? K : 1];
     int ki[SMALL ? K : 1];
@@ -59,6 +65,9 @@ __device__ __forceinline__ uint64_t select_mask(const RawFn& raw_at, int D, int 
             const int d = d0 - u;
             raw[u] = d >= 0 ? raw_at(d) : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u)
+            if (d0 - u >= 0) store_at(d0 - u, raw[u]);
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             const int d = d0 - u;
@@ -143,7 +152,7 @@ template <typename Tm, bool FROM_KEYS, int K>
 __global__ void __launch_bounds__(128)
 k_select(const Tm* __restrict__ M, const float* __restrict__ keys, int D, int h, int w, int k,
          uint8_t* __restrict__ S, uint64_t* __restrict__ mask_out, uint8_t* __restrict__ slots,
-         float* __restrict__ Gzero, int mode) {
+         float* __restrict__ Gzero, Tm* __restrict__ alphas, int mode) {
     const long long hw = (long long)h * w;
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= hw) return;
@@ -152,7 +161,10 @@ k_select(const Tm* __restrict__ M, const float* __restrict__ keys, int D, int h,
             if constexpr (FROM_KEYS) return __ldg(keys + (size_t)d * hw + p);
             else return RLStore<Tm>::load1(M + ((size_t)d * hw + p) * 4 + 3);
         },
-        D, k, mode);
+        D, k, mode,
+        [&](int d, float a) {
+            if (alphas) RLStore<Tm>::store1(alphas + (size_t)d * hw + p, a);
+        });
     write_selection(mk, D, k, hw, p, S, mask_out, slots, Gzero);
 }
 
@@ -198,8 +210,8 @@ template <typename Tm, int K, int LOG>
 __device__ __forceinline__ void pyramid_select_tile(const Tm* __restrict__ M, int D, int H, int W, int level,
                                                     Tm* __restrict__ Ml, int k, uint8_t* __restrict__ S,
                                                     uint8_t* __restrict__ slots, float* __restrict__ Gzero, int mode,
-                                                    long long p0,
-                                                    float (*alpha)[kTile]) {
+                                                    long long p0, float (*alpha)[kTile],
+                                                    Tm* __restrict__ alphas = nullptr) {
     const int h = H >> level, w = W >> level;
     const long long hw = (long long)h * w;
     // level 1: the loads of NB voxels (4 full-resolution voxels each) are issued together
@@ -221,6 +233,7 @@ __device__ __forceinline__ void pyramid_select_tile(const Tm* __restrict__ M, in
             if (i >= D * kTile || p >= hw) continue;
             RLStore<Tm>::store4(Ml + ((size_t)d * hw + p) * 4, v[b]);
             alpha[d][j] = RLStore<Tm>::round1(v[b].w);
+            if (alphas) RLStore<Tm>::store1(alphas + (size_t)d * hw + p, v[b].w);
         }
     }
     __syncthreads();
@@ -289,12 +302,11 @@ template <typename Tm, int K, int LOG>
 __global__ void __launch_bounds__(256)
 k_pyramid_select(const Tm* __restrict__ M, int D, int H, int W, int level, Tm* __restrict__ Ml, int k,
                  uint8_t* __restrict__ S, uint8_t* __restrict__ slots, float* __restrict__ Gzero, int mode,
-                 const float* __restrict__ images, int N,
-                 float* __restrict__ Il) {
+                 const float* __restrict__ images, int N, float* __restrict__ Il, Tm* __restrict__ alphas) {
     __shared__ float alpha[RL_DEV_MAX_PLANES][kTile];
     if (Il) level_image_means<LOG>(images, N, H, W, level, Il, (long long)blockIdx.x * kTile);
     pyramid_select_tile<Tm, K, LOG>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode,
-                                    (long long)blockIdx.x * kTile, alpha);
+                                    (long long)blockIdx.x * kTile, alpha, alphas);
 }
 
 // ------------------------------------------------------------------ batched selection
@@ -365,12 +377,12 @@ k_select_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restr
 
 template <typename Tm, bool FROM_KEYS>
 void launch_select_t(const void* M, const float* keys, int D, int h, int w, int k, uint8_t* S, uint64_t* mask,
-                     uint8_t* slots, float* Gzero, int mode, cudaStream_t s) {
+                     uint8_t* slots, float* Gzero, void* alphas, int mode, cudaStream_t s) {
     const long long hw = (long long)h * w;
     const int blocks = (int)((hw + 127) / 128);
 #define RL_SEL(KK)                                                                                          \
     k_select<Tm, FROM_KEYS, KK><<<blocks, 128, 0, s>>>((const Tm*)M, keys, D, h, w, k, S, mask, slots, Gzero, \
-                                                       mode)
+                                                       (Tm*)alphas, mode)
     switch (mode == 1 ? 1 : k) {
         case 1: RL_SEL(1); break;
         case 2: RL_SEL(2); break;
@@ -388,12 +400,12 @@ void launch_select_t(const void* M, const float* keys, int D, int h, int w, int 
 template <typename Tm, int LOG>
 void launch_pyramid_select_l(const Tm* M, int D, int H, int W, int level, Tm* Ml, int k, uint8_t* S,
                              uint8_t* slots, float* Gzero, int mode, cudaStream_t s,
-                             const float* images, int N, float* Il) {
+                             const float* images, int N, float* Il, void* alphas) {
     const long long hw = (long long)(H >> level) * (W >> level);
     const unsigned blocks = (unsigned)((hw + kTile - 1) / kTile);
 #define RL_PS(KK)                                                                                                 \
     k_pyramid_select<Tm, KK, LOG><<<blocks, 256, 0, s>>>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, \
-                                                         images, N, Il)
+                                                         images, N, Il, (Tm*)alphas)
     switch (mode == 1 ? 1 : k) {
         case 1: RL_PS(1); break;
         case 2: RL_PS(2); break;
@@ -411,13 +423,13 @@ void launch_pyramid_select_l(const Tm* M, int D, int H, int W, int level, Tm* Ml
 template <typename Tm>
 void launch_pyramid_select_t(const void* M, int D, int H, int W, int level, void* Ml, int k, uint8_t* S,
                              uint8_t* slots, float* Gzero, int mode, cudaStream_t s,
-                             const float* images, int N, float* Il) {
+                             const float* images, int N, float* Il, void* alphas) {
     if (level == 1)
-        launch_pyramid_select_l<Tm, 1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il);
+        launch_pyramid_select_l<Tm, 1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il, alphas);
     else if (level == 2)
-        launch_pyramid_select_l<Tm, 2>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il);
+        launch_pyramid_select_l<Tm, 2>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il, alphas);
     else
-        launch_pyramid_select_l<Tm, -1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il);
+        launch_pyramid_select_l<Tm, -1>((const Tm*)M, D, H, W, level, (Tm*)Ml, k, S, slots, Gzero, mode, s, images, N, Il, alphas);
 }
 
 __global__ void k_mask_to_slots(const uint64_t* __restrict__ mask, int D, int k, int hw,
@@ -454,32 +466,32 @@ __global__ void k_downsample_f32(const float* __restrict__ x, int P, int H, int 
 }  // namespace
 
 rl_status rl_launch_select(const void* M, rl_dtype dt, const float* keys, int D, int h, int w, int k, uint8_t* S,
-                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, int mode) {
+                           uint64_t* mask, uint8_t* slots, float* Gzero, cudaStream_t s, int mode, void* alphas) {
     if (keys) {
         RLTraceScope ts("select_keys", s);
-        launch_select_t<float, true>(nullptr, keys, D, h, w, k, S, mask, slots, Gzero, mode, s);
+        launch_select_t<float, true>(nullptr, keys, D, h, w, k, S, mask, slots, Gzero, alphas, mode, s);
     } else if (dt == RL_F32) {
         RLTraceScope ts("select_f32", s);
-        launch_select_t<float, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, mode, s);
+        launch_select_t<float, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, alphas, mode, s);
     } else {
         RLTraceScope ts("select_bf16", s);
-        launch_select_t<__nv_bfloat16, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, mode, s);
+        launch_select_t<__nv_bfloat16, false>(M, nullptr, D, h, w, k, S, mask, slots, Gzero, alphas, mode, s);
     }
     return rl_check_launch("select");
 }
 
 rl_status rl_launch_pyramid_select(const void* M, rl_dtype dt, int D, int H, int W, int level, void* Ml, int k,
                                    uint8_t* S, uint8_t* slots, float* Gzero, int mode,
-                                   cudaStream_t s, const float* images, int N, float* Il) {
+                                   cudaStream_t s, const float* images, int N, float* Il, void* alphas) {
     if (!images) Il = nullptr;
     if (dt == RL_F32) {
         RLTraceScope ts("pyramid_select_f32", s);
         launch_pyramid_select_t<float>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, s, images, N,
-                                       Il);
+                                       Il, alphas);
     } else {
         RLTraceScope ts("pyramid_select_bf16", s);
         launch_pyramid_select_t<__nv_bfloat16>(M, D, H, W, level, Ml, k, S, slots, Gzero, mode, s,
-                                               images, N, Il);
+                                               images, N, Il, alphas);
     }
     return rl_check_launch("pyramid_select");
 }

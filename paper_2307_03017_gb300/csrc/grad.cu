@@ -20,9 +20,13 @@
 // the latency of the gathers.  Warps whose samples all lie inside leave out the border tests.  With
 // many planes both passes take them in pairs, whose loads are in flight together, and pass 2 forms
 // T_d within a pair from the pair's stored one: half the shared memory, so that a launch of 64
-// planes keeps 32 warps an SM instead of 24, and its L1.  1920x1080, D = 64, 8 views, BF16, anchored:
-// 8.23 ms (one plane at a time 11.56 ms, groups of four 10.8 ms; at the start, with border tests in
-// every sample and a fenced loss reduction at the end of every block, 12.9 ms).
+// planes keeps 32 warps an SM instead of 24, and its L1.  Views that are pure shifts of the reference
+// (display and camera grids) have the same offset and weights at every pixel of a plane: a block
+// forms them once in FP64 and reads them from shared memory.  1920x1080, D = 64, 8 views, BF16:
+// 6.69 ms as shifts, 8.23 ms with anchored coordinates (one plane at a time 11.56 ms, groups of four
+// 10.8 ms; at the start, with border tests in every sample and a fenced loss reduction at the end of
+// every block, 12.9 ms).  Issue bound (78%): of the 197 instructions a sample left as shifts, 32
+// widen BF16, 16 blend and about 40 are the reductions of the taps.
 #include <type_traits>
 
 #include "rl_internal.h"
@@ -33,44 +37,124 @@ constexpr int kGradBX = 32, kGradBY = 4, kGradThreads = kGradBX * kGradBY;
 constexpr int kGroup = 2;          // planes whose samples are held together (grad_group, the batch)
 constexpr int kGradMinBlocks = 8;  // resident blocks the registers must then allow
 
+// How the taps of a sample are formed.
+constexpr int kPlain = 0, kAnchored = 1, kShifts = 2;
+
+// Views that are pure shifts of the reference: the offset p - q of plane d, the same for all pixels,
+// split in FP64 into an integer and a fraction.
+struct ShiftTable {
+    float4 w[RL_DEV_MAX_PLANES];   // the taps' weights
+    int off[RL_DEV_MAX_PLANES];    // iy W + ix
+    int ix[RL_DEV_MAX_PLANES], iy[RL_DEV_MAX_PLANES];
+    float fx[RL_DEV_MAX_PLANES], fy[RL_DEV_MAX_PLANES];
+
+    __device__ __forceinline__ RLTaps taps(int d, int qx, int qy) const {
+        RLTaps t;
+        t.ok = ix[d] != RL_PLANE_NONE;
+        t.x0 = qx + ix[d];
+        t.y0 = qy + iy[d];
+        t.fx = fx[d];
+        t.fy = fy[d];
+        return t;
+    }
+    // All four taps inside the plane.  The integer offset is monotone in d, so what holds for two
+    // planes holds for those between them.
+    __device__ __forceinline__ bool inside(int d, int qx, int qy, int H, int W) const {
+        return ix[d] != RL_PLANE_NONE && (unsigned)(qx + ix[d]) < (unsigned)(W - 1) &&
+               (unsigned)(qy + iy[d]) < (unsigned)(H - 1);
+    }
+};
+
+struct ShiftTap {
+    unsigned idx;  // voxel of the top-left tap within its plane
+    float4 w;
+};
+
+// Fills S for view `view`; every thread of the block calls it.
+__device__ __forceinline__ void shift_build(ShiftTable* S, const RLViews& V, int view, int D, int W, int tid) {
+    if (tid < D) {
+        const RLViewParam64& P = V.v64[view];
+        const double rho = V.rho64[tid];
+        const double kx = P.dcx + rho * (P.fxr * P.C[0]), ky = P.dcy + rho * (P.fyr * P.C[1]);
+        const bool ok = fabs(kx) < 1e9 && fabs(ky) < 1e9;
+        const double flx = floor(kx), fly = floor(ky);
+        S->ix[tid] = ok ? (int)flx : RL_PLANE_NONE;
+        S->iy[tid] = ok ? (int)fly : RL_PLANE_NONE;
+        S->off[tid] = ok ? (int)((unsigned)(int)fly * (unsigned)W + (unsigned)(int)flx) : 0;
+        S->fx[tid] = (float)(kx - flx);
+        S->fy[tid] = (float)(ky - fly);
+        S->w[tid] = rl_weights(S->fx[tid], S->fy[tid]);
+    }
+    __syncthreads();
+}
+
 // One block's tile of 32 x 4 view pixels of one view.  bid / nblocks index the block among
 // the launch's (or the batch item's) blocks for the loss partials.
-template <typename Tm, int GROUP, bool SPARSE, bool LOSS, bool ANCH>
+template <typename Tm, int GROUP, bool SPARSE, bool LOSS, int MODE>
 __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H, int W, const RLViews& views, int view,
                                           int qx, int qy, int tid, float* __restrict__ sT,
                                           const float* __restrict__ images, int img_level,
                                           const float* __restrict__ grad_out, const uint8_t* __restrict__ slots,
                                           float* __restrict__ G, float inv_n, float* __restrict__ partials,
                                           unsigned bid, unsigned nblocks) {
+    constexpr bool ANCH = MODE == kAnchored, SHIFT = MODE == kShifts;
     float lsum = 0.f;
     __shared__ RLAnchor sA;  // the tile's anchor: its centre pixel
+    __shared__ ShiftTable sS;
+    if (SHIFT) shift_build(&sS, views, view, D, W, tid);
     if (ANCH)
         rl_anchor_build(&sA, views, view, (qx & ~(kGradBX - 1)) + kGradBX / 2, qy - qy % kGradBY + kGradBY / 2, D,
                         W, tid, kGradThreads);
     const unsigned act = __ballot_sync(0xffffffffu, qx < W && qy < H);
     if (qx < W && qy < H) {
-        const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[view], qx, qy);
+        RLPixWarp<ANCH> w;
+        if constexpr (!SHIFT) w = rl_pix_warp<ANCH>(sA, views.v[view], qx, qy);
         const size_t plane = (size_t)H * W * 4;
-        const unsigned hw = (unsigned)(H * W), base = rl_fast_base(qx, qy, W);
-        // warps whose samples of every plane lie inside it skip the border tests
-        const bool fast = __all_sync(act, rl_chunk_inside<ANCH>(w, sA, views, 0, D - 1, qx, qy, H, W));
+        const unsigned hw = (unsigned)(H * W);
+        const unsigned base = SHIFT ? (unsigned)(qy * W + qx) : rl_fast_base(qx, qy, W);
+        // warps whose samples of every plane lie inside it skip the border tests; with shifts the whole
+        // tile row moves as one, and every kWalk planes are tested by themselves
+        constexpr int kWalk = 8, kPer = kWalk / GROUP;
+        const int n_chunks = (D + kWalk - 1) / kWalk;
+        unsigned chunks = 0u;
+        if constexpr (SHIFT) {
+            for (int c = 0; c < n_chunks; ++c) {
+                const int d0 = c * kWalk, d1 = min(d0 + kWalk, D) - 1;
+                if (__all_sync(act, sS.inside(d0, qx, qy, H, W) && sS.inside(d1, qx, qy, H, W))) chunks |= 1u << c;
+            }
+        } else {
+            chunks = __all_sync(act, rl_chunk_inside<ANCH>(w, sA, views, 0, D - 1, qx, qy, H, W)) ? 1u : 0u;
+        }
+        // the sample of plane d: top-left voxel and weights (inside), or footprint (anywhere)
+        const auto tap_inside = [&](int d) {
+            if constexpr (SHIFT) return ShiftTap{base + (unsigned)sS.off[d], sS.w[d]};
+            else return rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+        };
+        const auto weights = [](const auto& t) {
+            if constexpr (SHIFT) return t.w;
+            else return rl_weights(t.fx, t.fy);
+        };
+        const auto tap_any = [&](int d) {
+            if constexpr (SHIFT) return sS.taps(d, qx, qy);
+            else return w.taps(sA, d, views.rho[d], qx, qy);
+        };
         const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
         const int groups = (D + GROUP - 1) / GROUP;
         float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-        // the two kinds of warp take separate loops: a branch in every group costs 15%
-        const auto pass1 = [&](auto inside) {
+        // the two kinds take separate loops: a branch in every group costs 15%
+        const auto pass1 = [&](auto inside, int first, int end) {
 #pragma unroll 1
-            for (int j = groups - 1; j >= 0; --j) {
+            for (int j = end - 1; j >= first; --j) {
                 float4 m[GROUP];
 #pragma unroll
                 for (int i = GROUP - 1; i >= 0; --i) {
                     const int d = j * GROUP + i, dc = GROUP == 1 ? d : min(d, D - 1);
                     if constexpr (decltype(inside)::value) {
-                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, dc, base, W);
+                        const auto t = tap_inside(dc);
                         m[i] = RL_IN((long long)t.idx + W + 1, hw)
-                                   ? rl_sample_at(M, (unsigned)dc * hw + t.idx, W, t.fx, t.fy) : none;
+                                   ? rl_sample_at(M, (unsigned)dc * hw + t.idx, W, weights(t)) : none;
                     } else {
-                        m[i] = rl_sample_fast(M + dc * plane, H, W, w.taps(sA, dc, views.rho[dc], qx, qy));
+                        m[i] = rl_sample_fast(M + dc * plane, H, W, tap_any(dc));
                     }
                     if (GROUP > 1 && d >= D) m[i] = none;  // beyond the last plane
                 }
@@ -85,8 +169,17 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
                 }
             }
         };
-        if (fast) pass1(std::true_type());
-        else pass1(std::false_type());
+        if constexpr (SHIFT) {
+#pragma unroll 1
+            for (int c = n_chunks - 1; c >= 0; --c) {
+                if ((chunks >> c) & 1u) pass1(std::true_type(), c * kPer, min((c + 1) * kPer, groups));
+                else pass1(std::false_type(), c * kPer, min((c + 1) * kPer, groups));
+            }
+        } else if (chunks) {
+            pass1(std::true_type(), 0, groups);
+        } else {
+            pass1(std::false_type(), 0, groups);
+        }
         float r0, r1, r2;
         if (LOSS) {
             // source image at this level: mean of the 2^l x 2^l full-resolution block
@@ -117,27 +210,27 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
         }
         float b0 = 0.f, b1 = 0.f, b2 = 0.f;
         const unsigned ng = views.gplanes ? (unsigned)views.gplanes : (unsigned)D;  // checked in debug builds
-        const auto pass2 = [&](auto inside) {
+        const auto pass2 = [&](auto inside, int first, int end) {
 #pragma unroll 1
-            for (int j = 0; j < groups; ++j) {
+            for (int j = first; j < end; ++j) {
                 float4 m[GROUP];
                 float Td[GROUP];
                 unsigned word[GROUP];
-                RLFastTap tap[GROUP];
+                decltype(tap_inside(0)) tap[GROUP];
 #pragma unroll
                 for (int i = GROUP - 1; i >= 0; --i) {
                     const int d = j * GROUP + i, dc = GROUP == 1 ? d : min(d, D - 1);
                     if constexpr (decltype(inside)::value) {
-                        tap[i] = rl_fast_tap<ANCH>(w, sA, views, dc, base, W);
+                        tap[i] = tap_inside(dc);
                         const unsigned e = (unsigned)dc * hw + tap[i].idx;
                         m[i] = none;
                         word[i] = 0xFFFFFFFFu;
                         if (RL_IN((long long)tap[i].idx + W + 1, hw)) {
                             if (SPARSE) word[i] = rl_slot_word(slots, e, W);
-                            m[i] = rl_sample_at(M, e, W, tap[i].fx, tap[i].fy);
+                            m[i] = rl_sample_at(M, e, W, weights(tap[i]));
                         }
                     } else {
-                        m[i] = rl_sample_fast(M + dc * plane, H, W, w.taps(sA, dc, views.rho[dc], qx, qy));
+                        m[i] = rl_sample_fast(M + dc * plane, H, W, tap_any(dc));
                     }
                     if (GROUP > 1 && d >= D) m[i] = none;
                 }
@@ -157,11 +250,11 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
                                         Td[i] * fmaf(m[i].x - b0, r0, fmaf(m[i].y - b1, r1, (m[i].z - b2) * r2)));
                         if constexpr (decltype(inside)::value) {
                             // a pair forms its taps again (they cost registers); a single plane keeps them
-                            const RLFastTap t = GROUP == 1 ? tap[i] : rl_fast_tap<ANCH>(w, sA, views, d, base, W);
+                            const auto t = GROUP == 1 ? tap[i] : tap_inside(d);
                             rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W,
-                                                  t.fx, t.fy, g, ng);
+                                                  weights(t), g, ng);
                         } else {
-                            const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
+                            const RLTaps t = tap_any(d);
                             if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);
                         }
                     }
@@ -172,8 +265,17 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
                 }
             }
         };
-        if (fast) pass2(std::true_type());
-        else pass2(std::false_type());
+        if constexpr (SHIFT) {
+#pragma unroll 1
+            for (int c = 0; c < n_chunks; ++c) {
+                if ((chunks >> c) & 1u) pass2(std::true_type(), c * kPer, min((c + 1) * kPer, groups));
+                else pass2(std::false_type(), c * kPer, min((c + 1) * kPer, groups));
+            }
+        } else if (chunks) {
+            pass2(std::true_type(), 0, groups);
+        } else {
+            pass2(std::false_type(), 0, groups);
+        }
     }
     if (LOSS) {
         __shared__ float red[kGradThreads / 32];
@@ -188,14 +290,14 @@ __device__ __forceinline__ void grad_tile(const Tm* __restrict__ M, int D, int H
     }
 }
 
-template <typename Tm, int GROUP, bool SPARSE, bool LOSS, bool ANCH>
+template <typename Tm, int GROUP, bool SPARSE, bool LOSS, int MODE>
 __global__ void __launch_bounds__(kGradThreads, GROUP == 1 ? 10 : kGradMinBlocks)
 k_grad(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views,
        const float* __restrict__ images, int img_level, const float* __restrict__ grad_out,
        const uint8_t* __restrict__ slots, float* __restrict__ G, float inv_n, float* __restrict__ partials) {
     extern __shared__ float sT[];  // [ceil(D / GROUP)][kGradThreads]
     // view-fastest block order: the N views of a tile run together and share M through L2
-    grad_tile<Tm, GROUP, SPARSE, LOSS, ANCH>(M, D, H, W, views, blockIdx.x, blockIdx.y * kGradBX + threadIdx.x,
+    grad_tile<Tm, GROUP, SPARSE, LOSS, MODE>(M, D, H, W, views, blockIdx.x, blockIdx.y * kGradBX + threadIdx.x,
                                 blockIdx.z * kGradBY + threadIdx.y, threadIdx.y * kGradBX + threadIdx.x, sT, images,
                                 img_level, grad_out, slots, G, inv_n, partials,
                                 blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z),
@@ -229,8 +331,8 @@ k_grad_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __restric
                                              it.level ? it.Il : it.images, 0, nullptr, it.slots, it.G, it.inv_n,    \
                                              it.partials,                                                           \
                                              local, it.grad_units)
-        if (it.views.anchored) RL_GB(true);
-        else RL_GB(false);
+        if (it.views.anchored) RL_GB(kAnchored);
+        else RL_GB(kPlain);
 #undef RL_GB
         __syncthreads();  // sT is reused by the next unit
     }
@@ -256,9 +358,11 @@ void launch_grad_t(const void* M, int D, int H, int W, const RLViews& views, con
                    dim3 grid, cudaStream_t s) {
     const int group = grad_group(D, sizeof(Tm) == 4);
     const size_t smem = (size_t)((D + group - 1) / group) * kGradThreads * sizeof(float);
-    auto kern = group == 1
-                    ? (views.anchored ? k_grad<Tm, 1, SPARSE, LOSS, true> : k_grad<Tm, 1, SPARSE, LOSS, false>)
-                    : (views.anchored ? k_grad<Tm, kGroup, SPARSE, LOSS, true> : k_grad<Tm, kGroup, SPARSE, LOSS, false>);
+#define RL_MODE(GR) (views.shifts ? k_grad<Tm, GR, SPARSE, LOSS, kShifts>            \
+                     : views.anchored ? k_grad<Tm, GR, SPARSE, LOSS, kAnchored>   \
+                                      : k_grad<Tm, GR, SPARSE, LOSS, kPlain>)
+    auto kern = group == 1 ? RL_MODE(1) : RL_MODE(kGroup);
+#undef RL_MODE
     kern<<<grid, dim3(kGradBX, kGradBY), smem, s>>>((const Tm*)M, D, H, W, views, images, img_level, grad_out, slots, G,
                                                     inv_n, partials);
 }
@@ -274,7 +378,7 @@ size_t rl_grad_num_blocks(int H, int W, int N) {
 rl_status rl_launch_grad(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                          const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G,
                          float inv_n, float* partials, int* nblocks, cudaStream_t s) {
-    if (rl_grad_path(H, W, views.n, D, views.anchored != 0, slots != nullptr) != 2)
+    if (rl_grad_path(H, W, views.n, D, views.anchored != 0, views.shifts != 0, slots != nullptr) != 2)
         return rl_launch_grad_pp(M, dt, D, H, W, views, mode_loss, images, img_level, grad_out, slots, G, inv_n,
                                  partials, nblocks, s);
     const int tiles_x = (W + kGradBX - 1) / kGradBX, tiles_y = (H + kGradBY - 1) / kGradBY;

@@ -214,7 +214,7 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
 #pragma unroll
         for (int i = C - 1; i >= 0; --i) {
             const int d = FULL ? d0 + i : d0 + min(i, n - 1);
-            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
+            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
             m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             word[i] = 0xFFFFFFFFu;
             if (RL_IN((long long)t.idx + W + 1, hw)) {
@@ -322,9 +322,9 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
                     g.z = gc * r2;
                     g.w = Td * fmaf(mi.x - b0, r0, fmaf(mi.y - b1, r1, (mi.z - b2) * r2));
                     if (fast) {  // the taps are formed again: keeping them costs registers, and warps
-                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d, base, W);
-                        rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W, t.fx,
-                                              t.fy, g, ng);
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                        rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W,
+                                              rl_weights(t.fx, t.fy), g, ng);
                     } else {
                         const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
                         if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);

@@ -368,6 +368,7 @@ rl_status make_views(const rl_mpi* m, const rl_camera* cams, int n, int level, R
                            "(1 + e_z <= 0.05); such views are not supported",
                            i);
     }
+    v.shifts = rl_views_are_shifts(v);
     return RL_OK;
 }
 

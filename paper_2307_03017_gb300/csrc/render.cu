@@ -60,7 +60,7 @@ k_render(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ 
             float4 m[kRenderGroup];
 #pragma unroll
             for (int i = 0; i < kRenderGroup; ++i) {
-                const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d - i, base, W);
+                const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d - i, views.rho[d - i], base, W);
                 m[i] = RL_IN((long long)t.idx + W + 1, hw)
                            ? rl_sample_at(M, (unsigned)(d - i) * hw + t.idx, W, t.fx, t.fy)
                            : make_float4(0.f, 0.f, 0.f, 0.f);

@@ -77,6 +77,7 @@ struct RLViews {
     double rho64[RL_DEV_MAX_PLANES];
     RLViewParam64 v64[RL_DEV_MAX_VIEWS];
     int gplanes;  // planes of the gradient buffer a launch scatters into (0: D); debug-build bounds checks
+    int shifts;   // 1: every view is a pure shift of the reference (rl_views_are_shifts)
 };
 
 // ------------------------------------------------------------------ batch work tables
@@ -538,8 +539,8 @@ __device__ __forceinline__ unsigned rl_fast_base(int qx, int qy, int W) {
 }
 
 template <bool ANCH>
-__device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const RLAnchor& A, const RLViews& views,
-                                                 int d, unsigned base, int W) {
+__device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const RLAnchor& A, int d, float rho,
+                                                 unsigned base, int W) {
     float sx, sy;
     if constexpr (ANCH) {
         const RLPlaneF k = A.f[d];
@@ -547,7 +548,6 @@ __device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const
         sy = k.fy + fmaf(k.rho, w.w.dby, w.w.day);
         base += (unsigned)k.off;
     } else {
-        const float rho = views.rho[d];
         sx = fmaf(rho, w.w.bx, w.w.ax);
         sy = fmaf(rho, w.w.by, w.w.ay);
     }
@@ -588,29 +588,38 @@ __device__ __forceinline__ bool rl_chunk_inside(const RLPixWarp<ANCH>& w, const 
            fminf(y0, y1) >= 1.f && fmaxf(y0, y1) < (float)(H - 2);
 }
 
+// Weights of a sample's taps (x: left upper, y: right upper, z: left lower, w: right lower).
+__device__ __forceinline__ float4 rl_weights(float fx, float fy) {
+    const float gx = 1.f - fx, gy = 1.f - fy;
+    return make_float4(gx * gy, fx * gy, gx * fy, fx * fy);
+}
+
 // The four taps of a sample blended with packed FP32x2 FMAs (the order of rl_sample).
 __device__ __forceinline__ float4 rl_blend(const float4& v00, const float4& v10, const float4& v01, const float4& v11,
-                                           float fx, float fy) {
-    const float gx = 1.f - fx, gy = 1.f - fy;
-    const float w00 = gx * gy, w10 = fx * gy, w01 = gx * fy, w11 = fx * fy;
-    float2 lo = __fmul2_rn(make_float2(w00, w00), make_float2(v00.x, v00.y));
-    float2 hi = __fmul2_rn(make_float2(w00, w00), make_float2(v00.z, v00.w));
-    lo = __ffma2_rn(make_float2(w10, w10), make_float2(v10.x, v10.y), lo);
-    hi = __ffma2_rn(make_float2(w10, w10), make_float2(v10.z, v10.w), hi);
-    lo = __ffma2_rn(make_float2(w01, w01), make_float2(v01.x, v01.y), lo);
-    hi = __ffma2_rn(make_float2(w01, w01), make_float2(v01.z, v01.w), hi);
-    lo = __ffma2_rn(make_float2(w11, w11), make_float2(v11.x, v11.y), lo);
-    hi = __ffma2_rn(make_float2(w11, w11), make_float2(v11.z, v11.w), hi);
+                                           const float4& w) {
+    float2 lo = __fmul2_rn(make_float2(w.x, w.x), make_float2(v00.x, v00.y));
+    float2 hi = __fmul2_rn(make_float2(w.x, w.x), make_float2(v00.z, v00.w));
+    lo = __ffma2_rn(make_float2(w.y, w.y), make_float2(v10.x, v10.y), lo);
+    hi = __ffma2_rn(make_float2(w.y, w.y), make_float2(v10.z, v10.w), hi);
+    lo = __ffma2_rn(make_float2(w.z, w.z), make_float2(v01.x, v01.y), lo);
+    hi = __ffma2_rn(make_float2(w.z, w.z), make_float2(v01.z, v01.w), hi);
+    lo = __ffma2_rn(make_float2(w.w, w.w), make_float2(v11.x, v11.y), lo);
+    hi = __ffma2_rn(make_float2(w.w, w.w), make_float2(v11.z, v11.w), hi);
     return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
 
 // Sample inside the plane: voxel e of the MPI is the top-left tap.
 template <typename Tm>
-__device__ __forceinline__ float4 rl_sample_at(const Tm* __restrict__ M, unsigned e, int W, float fx, float fy) {
+__device__ __forceinline__ float4 rl_sample_at(const Tm* __restrict__ M, unsigned e, int W, const float4& w) {
     const Tm* p = M + (size_t)e * 4u;
     const Tm* q = M + (size_t)(e + (unsigned)W) * 4u;
     return rl_blend(RLStore<Tm>::load4(p), RLStore<Tm>::load4(p + 4), RLStore<Tm>::load4(q), RLStore<Tm>::load4(q + 4),
-                    fx, fy);
+                    w);
+}
+
+template <typename Tm>
+__device__ __forceinline__ float4 rl_sample_at(const Tm* __restrict__ M, unsigned e, int W, float fx, float fy) {
+    return rl_sample_at(M, e, W, rl_weights(fx, fy));
 }
 
 // Adds wt (gl, gh) to one voxel of the gradient.
@@ -631,23 +640,22 @@ __device__ __forceinline__ unsigned rl_slot_word(const uint8_t* __restrict__ slo
 // voxel e of the MPI.  SPARSE: only into the taps that have a slot in the compact gradient.
 template <bool SPARSE>
 __device__ __forceinline__ void rl_scatter_at(float* __restrict__ G, unsigned word, unsigned d, unsigned p, unsigned e,
-                                              unsigned hw, int W, float fx, float fy, float4 g, unsigned ng) {
+                                              unsigned hw, int W, const float4& w, float4 g, unsigned ng) {
     float4* G4 = reinterpret_cast<float4*>(G);
-    const float gx = 1.f - fx, gy = 1.f - fy;
     const float2 gl = make_float2(g.x, g.y), gh = make_float2(g.z, g.w);
     if constexpr (SPARSE) {
         if (word == 0xFFFFFFFFu) return;
         const unsigned s00 = word & 255u, s10 = (word >> 8) & 255u, s01 = (word >> 16) & 255u, s11 = word >> 24;
-        if (s00 != RL_SLOT_NONE && RL_IN(s00, ng)) rl_add_tap(G4, s00 * hw + p, gx * gy, gl, gh);
-        if (s10 != RL_SLOT_NONE && RL_IN(s10, ng)) rl_add_tap(G4, s10 * hw + p + 1u, fx * gy, gl, gh);
-        if (s01 != RL_SLOT_NONE && RL_IN(s01, ng)) rl_add_tap(G4, s01 * hw + p + (unsigned)W, gx * fy, gl, gh);
-        if (s11 != RL_SLOT_NONE && RL_IN(s11, ng)) rl_add_tap(G4, s11 * hw + p + (unsigned)W + 1u, fx * fy, gl, gh);
+        if (s00 != RL_SLOT_NONE && RL_IN(s00, ng)) rl_add_tap(G4, s00 * hw + p, w.x, gl, gh);
+        if (s10 != RL_SLOT_NONE && RL_IN(s10, ng)) rl_add_tap(G4, s10 * hw + p + 1u, w.y, gl, gh);
+        if (s01 != RL_SLOT_NONE && RL_IN(s01, ng)) rl_add_tap(G4, s01 * hw + p + (unsigned)W, w.z, gl, gh);
+        if (s11 != RL_SLOT_NONE && RL_IN(s11, ng)) rl_add_tap(G4, s11 * hw + p + (unsigned)W + 1u, w.w, gl, gh);
     } else {
         if (!RL_IN(d, ng)) return;
-        rl_add_tap(G4, e, gx * gy, gl, gh);
-        rl_add_tap(G4, e + 1u, fx * gy, gl, gh);
-        rl_add_tap(G4, e + (unsigned)W, gx * fy, gl, gh);
-        rl_add_tap(G4, e + (unsigned)W + 1u, fx * fy, gl, gh);
+        rl_add_tap(G4, e, w.x, gl, gh);
+        rl_add_tap(G4, e + 1u, w.y, gl, gh);
+        rl_add_tap(G4, e + (unsigned)W, w.z, gl, gh);
+        rl_add_tap(G4, e + (unsigned)W + 1u, w.w, gl, gh);
     }
 }
 

@@ -40,13 +40,13 @@ int rl_kernel_path(int H, int W, int nviews) {
     return (long long)H * W * nviews < (1ll << 19) ? 3 : 2;
 }
 
-int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool sparse) {
+int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bool sparse) {
     const int p = g_path.load(std::memory_order_relaxed);
     if (p != 0) return p >= 3 ? 3 : p;
     if (H > 2 * 65535) return 2;  // beyond the plane-parallel grid
     const long long pixel_views = (long long)H * W * nviews;
-    if (pixel_views < (1ll << 19)) return 3;
-    if (anchored) return 2;
+    if (pixel_views < (1ll << (shifts ? 18 : 19))) return 3;
+    if (anchored || shifts) return 2;
     return sparse ? (D <= 32 || pixel_views < (1ll << 20) ? 3 : 2) : (D <= 32 && pixel_views < (1ll << 20) ? 3 : 2);
 }
 

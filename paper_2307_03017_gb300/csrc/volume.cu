@@ -97,7 +97,7 @@ k_view_alpha(const Tm* __restrict__ M, int D, int H, int W, const __grid_constan
             float a[kAlphaGroup];
 #pragma unroll
             for (int i = 0; i < kAlphaGroup; ++i) {
-                const RLFastTap t = rl_fast_tap<ANCH>(w, sA, views, d - i, base, W);
+                const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d - i, views.rho[d - i], base, W);
                 a[i] = 0.f;
                 if (!RL_IN((long long)t.idx + W + 1, hw)) continue;
                 const Tm* p = M + (size_t)((unsigned)(d - i) * hw + t.idx) * CH;

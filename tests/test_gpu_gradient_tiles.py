@@ -45,6 +45,24 @@ def test_gradient_at_tile_and_chunk_edges(rl, H, W, D, N, f, path):
     assert np.abs(G.cpu().numpy() - g_o).max() <= TOL32
 
 
+# views that are pure shifts read their taps from a table: shifts beyond the image, odd widths, both
+# numbers of planes at a time and their remainders
+@pytest.mark.parametrize("H,W,D,f", [(9, 64, 5, None), (7, 33, 33, None), (12, 97, 50, 300.0), (6, 40, 1, None)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_gradient_of_shifted_views(rl, H, W, D, f, dtype):
+    sc = sg.make_scene(12, H, W, D, 8, n_layers=(1, 2), src_poses="grid4x2", novel="none", f=f)
+    rl.reallife_set_kernel_path(2)
+    try:
+        m = rl.make_mpi(_dev(sc.coarse_mpi, dtype), sc.near, sc.far, sc.ref)
+        loss, G = rl.reallife_loss_grad(m, _dev(sc.images), sc.src)
+    finally:
+        rl.reallife_set_kernel_path(0)
+    stored = m.data.float().cpu().numpy()
+    L_o, g_o, _ = oracle.loss_grad(stored, sc.near, sc.far, sc.ref, sc.src, sc.images)
+    assert abs(loss.item() - L_o) <= 1e-5 * max(L_o, 1e-3)
+    assert np.abs(G.cpu().numpy() - g_o).max() <= TOL32
+
+
 # the two gradient families a batch may take: the automatic rule's small and large batches
 @pytest.mark.parametrize("H,W,n", [(24, 34, 3), (256, 352, 3)])
 def test_batch_family_by_size_equals_single_steps(rl, H, W, n):

@@ -35,17 +35,17 @@ int rl_kernel_path(int H, int W, int nviews);
 // The same for the gradient of D planes (sparse: compact).  Automatic, by measured times:
 //  - fewer than 2^19 pixel-views: plane-parallel, which gathers each sample once (64x48, 2 views,
 //    D = 32: 13 against 51 us; 256x192, 8 views, D = 64: 233 against 289 us);
-//  - pure shifts, from 2^18 pixel-views on: per-pixel, which reads their taps from a table (512x384, 2
-//    views, D = 32, BF16: 108 against 168 us; 4 views: 194 against 206; 256x192, 4 views: 83 against 66);
+//  - pure shifts with a compact gradient, from 2^18 pixel-views on: per-pixel, which reads their taps
+//    from a table (512x384, 2 views, D = 32, BF16: 108 against 168 us; 256x192, 4 views: 83
+//    against 66);
 //  - anchored coordinates: per-pixel, since a plane-parallel block repeats the FP64 set-up of the
 //    anchors for every 32 pixels, a per-pixel one for every 128 (1024x768, 4 views, D = 64, BF16:
 //    2507 against 1710 us);
 //  - compact: plane-parallel up to 32 planes (512x384, 4 views, BF16: 206 against 246 us; 700x768:
 //    545 against 593) or 2^20 pixel-views (512x384, D = 64: 442 against 465); beyond, the chunk
 //    exchange of sixteen warps costs more than the second gather (700x768, D = 64: 1178 against 1112);
-//  - dense: every tap is a reduction and L2 the bound; plane-parallel only up to 32 planes and 2^20
-//    pixel-views (500x375, 4 views, D = 32: 284 against 290 us; 960x540, 2 views, D = 64: 963
-//    against 826; 900x540, 4 views, D = 20: 420 against 392).
+//  - dense: plane-parallel, whose warps join their lanes' shared taps (500x375, 4 views, D = 32: 226
+//    against 290 us; 960x540, 2 views, D = 64: 793 against 828).
 int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bool sparse);
 // The gradient family of a batched step of so many pixel-views in all: per-pixel gather, whose long
 // units hide the cost of fetching them (eight requests of 2 to 50 M samples: 2484 us against 3475 us

@@ -45,9 +45,10 @@ int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bo
     if (p != 0) return p >= 3 ? 3 : p;
     if (H > 2 * 65535) return 2;  // beyond the plane-parallel grid
     const long long pixel_views = (long long)H * W * nviews;
-    if (pixel_views < (1ll << (shifts ? 18 : 19))) return 3;
-    if (anchored || shifts) return 2;
-    return sparse ? (D <= 32 || pixel_views < (1ll << 20) ? 3 : 2) : (D <= 32 && pixel_views < (1ll << 20) ? 3 : 2);
+    if (sparse && shifts && pixel_views >= (1ll << 18)) return 2;
+    if (pixel_views < (1ll << 19)) return 3;
+    if (anchored) return 2;
+    return !sparse || D <= 32 || pixel_views < (1ll << 20) ? 3 : 2;
 }
 
 int rl_batch_grad_path(long long pixel_views) {

@@ -33,11 +33,11 @@ unsigned int* rl_device_status_ptr();
 // and per-pixel gather otherwise.
 int rl_kernel_path(int H, int W, int nviews);
 // The same for the gradient of D planes (sparse: compact).  Automatic, by measured times:
-//  - fewer than 2^19 pixel-views: plane-parallel, which gathers each sample once (64x48, 2 views,
+//  - else fewer than 2^19 pixel-views: plane-parallel, which gathers each sample once (64x48, 2 views,
 //    D = 32: 13 against 51 us; 256x192, 8 views, D = 64: 233 against 289 us);
-//  - pure shifts with a compact gradient, from 2^18 pixel-views on: per-pixel, which reads their taps
-//    from a table (512x384, 2 views, D = 32, BF16: 108 against 168 us; 256x192, 4 views: 83
-//    against 66);
+//  - pure shifts with a compact gradient, from 2^17 pixel-views on: per-pixel, whose kernel for them
+//    shares taps between two pixels and forms no coordinates (256x192, 4 views, D = 32, FP32: 51
+//    against 64 us; 512x384, 4 views, BF16: 175 against 206);
 //  - anchored coordinates: per-pixel, since a plane-parallel block repeats the FP64 set-up of the
 //    anchors for every 32 pixels, a per-pixel one for every 128 (1024x768, 4 views, D = 64, BF16:
 //    2507 against 1710 us);

@@ -45,7 +45,7 @@ int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bo
     if (p != 0) return p >= 3 ? 3 : p;
     if (H > 2 * 65535) return 2;  // beyond the plane-parallel grid
     const long long pixel_views = (long long)H * W * nviews;
-    if (sparse && shifts && pixel_views >= (1ll << 18)) return 2;
+    if (sparse && shifts && pixel_views >= (1ll << 17)) return 2;
     if (pixel_views < (1ll << 19)) return 3;
     if (anchored) return 2;
     return !sparse || D <= 32 || pixel_views < (1ll << 20) ? 3 : 2;

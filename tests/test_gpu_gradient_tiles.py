@@ -45,8 +45,8 @@ def test_gradient_at_tile_and_chunk_edges(rl, H, W, D, N, f, path):
     assert np.abs(G.cpu().numpy() - g_o).max() <= TOL32
 
 
-# views that are pure shifts read their taps from a table: shifts beyond the image, odd widths, both
-# numbers of planes at a time and their remainders
+# views that are pure shifts share taps between two rows: shifts beyond the image, taps left of and
+# above the first voxel of all (plane 0, column and row -1), odd widths and heights, a single plane
 @pytest.mark.parametrize("H,W,D,f", [(9, 64, 5, None), (7, 33, 33, None), (12, 97, 50, 300.0), (6, 40, 1, None)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_gradient_of_shifted_views(rl, H, W, D, f, dtype):
@@ -55,12 +55,18 @@ def test_gradient_of_shifted_views(rl, H, W, D, f, dtype):
     try:
         m = rl.make_mpi(_dev(sc.coarse_mpi, dtype), sc.near, sc.far, sc.ref)
         loss, G = rl.reallife_loss_grad(m, _dev(sc.images), sc.src)
+        k = min(3, D)
+        S, mask = rl.reallife_select(m, k)
+        loss_s, Gs = rl.reallife_loss_grad(m, _dev(sc.images), sc.src, mask=mask, k=k)
     finally:
         rl.reallife_set_kernel_path(0)
     stored = m.data.float().cpu().numpy()
     L_o, g_o, _ = oracle.loss_grad(stored, sc.near, sc.far, sc.ref, sc.src, sc.images)
     assert abs(loss.item() - L_o) <= 1e-5 * max(L_o, 1e-3)
     assert np.abs(G.cpu().numpy() - g_o).max() <= TOL32
+    assert abs(loss_s.item() - L_o) <= 1e-5 * max(L_o, 1e-3)
+    want = np.take_along_axis(g_o, S.cpu().numpy().astype(np.int64)[..., None], axis=0)
+    assert np.abs(Gs.cpu().numpy() - want).max() <= TOL32
 
 
 # the two gradient families a batch may take: the automatic rule's small and large batches

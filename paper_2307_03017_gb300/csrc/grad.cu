@@ -21,7 +21,7 @@
 // many planes both passes take them in pairs, whose loads are in flight together, and pass 2 forms
 // T_d within a pair from the pair's stored one: half the shared memory, so that a launch of 64
 // planes keeps 32 warps an SM instead of 24, and its L1.  1920x1080, D = 64, 8
-// views, BF16, anchored: 8.23 ms (one plane at a time 11.56 ms, groups of four 10.8 ms; at the start,
+// views, BF16, anchored: 8.23 ms (one plane at a time 11.56 ms, groups of four 10.8 ms; before,
 // with border tests in every sample and a fenced loss reduction at the end of every block, 12.9 ms).
 // Views that are pure shifts of the reference take a kernel of their own (k_grad_shift).
 #include <type_traits>

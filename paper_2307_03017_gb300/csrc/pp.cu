@@ -175,10 +175,10 @@ __device__ __forceinline__ PPPos pp_pos(int H, int W, int view, int bx, int by, 
 
 // Dense transpose of a warp's samples inside plane d, one voxel e (top-left tap) a lane: where a lane's
 // left taps are its neighbour's right ones, the neighbour's share comes by shuffles and one reduction
-// adds both, so most voxels of a row take one reduction instead of two.  The reductions are the bound
-// of the dense gradient (L1, ten wavefronts each; L2): 4 views of 500x375, D = 32, FP32: 226 us, 286 us
-// without the joining.  Lanes outside `act` and lanes with live = false
-// pass g = 0.
+// adds both, so most voxels of a row take one reduction instead of two.  4 views of 500x375, D = 32,
+// FP32: 224 us, 286 us without the joining, whose reductions were the bound (L1, ten wavefronts each;
+// L2).  Now issue is (68%; L1 66%, L2 47%): joining the row below as well costs 237 us.  Lanes outside
+// `act` and lanes with live = false pass g = 0.
 __device__ __forceinline__ void join_taps(float* __restrict__ G, unsigned act, int lane, bool live, unsigned d,
                                           unsigned e, int W, float fx, float fy, float4 g, unsigned ng) {
     float4* G4 = reinterpret_cast<float4*>(G);

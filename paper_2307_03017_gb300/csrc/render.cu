@@ -8,10 +8,11 @@
 // What bounds it: instruction issue (1920x1080, D = 64, BF16, anchored: 78% of the issue slots at
 // 83 instructions a sample before).  A warp whose samples of the nearest and the farthest plane lie
 // inside the planes has all of them inside, so it leaves out the border tests and takes the fast
-// coordinates of rl_common.cuh, two planes at a time: 13.6 against 17.0 ms for 45 such views, 82
-// against 86 us for 4 rotated 500x375 views, D = 32, FP32 (one plane at a time 14.7 ms, four 14.5).  Views that are pure shifts of the reference (no
-// rotation, no depth offset, same focal lengths) take a kernel that computes each plane's
-// shift and weights once per block and renders four pixels of a column per thread, loading
+// coordinates of rl_common.cuh, two planes at a time: 13.2 against 17.0 ms for 45 such views, 82
+// against 86 us for 4 rotated 500x375 views, D = 32, FP32 (13.6 ms without the packed arithmetic of
+// positions and weights; without it too, one plane at a time 14.7 ms, four 14.5).  Views that are pure
+// shifts of the reference (no rotation, no depth offset, same focal lengths) take a kernel that
+// computes each plane's shift and weights once per block and renders four pixels of a column per thread, loading
 // each tap row once.
 #include "rl_internal.h"
 
@@ -62,7 +63,7 @@ k_render(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ 
             for (int i = 0; i < kRenderGroup; ++i) {
                 const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d - i, views.rho[d - i], base, W);
                 m[i] = RL_IN((long long)t.idx + W + 1, hw)
-                           ? rl_sample_at(M, (unsigned)(d - i) * hw + t.idx, W, t.fx, t.fy)
+                           ? rl_sample_at(M, (unsigned)(d - i) * hw + t.idx, W, rl_weights_packed(t.fx, t.fy))
                            : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll

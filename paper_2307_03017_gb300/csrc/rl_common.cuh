@@ -524,10 +524,18 @@ __device__ __forceinline__ float4 rl_sample_fast(const Tm* __restrict__ plane, i
 // Fast coordinates of a sample known to lie inside the plane: the floor comes from an addition
 // rounded towards minus infinity to a multiple of one (exact for |s| < 2^22), whose mantissa is
 // also the integer part, so that a sample needs no conversion instruction and one multiply-add
-// forms its voxel index.  Same values as rl_taps / rl_anchor_taps.
+// forms its voxel index.  Same values as rl_taps / rl_anchor_taps.  Both coordinates go through
+// packed FP32x2 instructions, each half rounded as a scalar one, which halves the arithmetic of a
+// position: 45 views of 1920x1080, D = 64, BF16: 13.35 against 13.63 ms; batched gradient 2.26
+// against 2.30 ms; view alpha weights 53 against 55 us; the other gradients within 1%.
 #define RL_FLOOR_MAGIC 12582912.f  // 1.5 * 2^23
 #define RL_FLOOR_BITS 0x4B400000u
 #define RL_FAST_EXTENT (1 << 20)       // image sides for which the fast coordinates are exact
+
+// a - b, both halves (one rounding each, as a subtraction)
+__device__ __forceinline__ float2 rl_minus2(float2 a, float2 b) {
+    return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
 
 struct RLFastTap {
     unsigned idx;  // voxel of the top-left tap within its plane
@@ -541,21 +549,21 @@ __device__ __forceinline__ unsigned rl_fast_base(int qx, int qy, int W) {
 template <bool ANCH>
 __device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const RLAnchor& A, int d, float rho,
                                                  unsigned base, int W) {
-    float sx, sy;
+    float2 s;
     if constexpr (ANCH) {
         const RLPlaneF k = A.f[d];
-        sx = k.fx + fmaf(k.rho, w.w.dbx, w.w.dax);
-        sy = k.fy + fmaf(k.rho, w.w.dby, w.w.day);
+        s = __ffma2_rn(make_float2(k.rho, k.rho), make_float2(w.w.dbx, w.w.dby), make_float2(w.w.dax, w.w.day));
+        s = __fadd2_rn(make_float2(k.fx, k.fy), s);
         base += (unsigned)k.off;
     } else {
-        sx = fmaf(rho, w.w.bx, w.w.ax);
-        sy = fmaf(rho, w.w.by, w.w.ay);
+        s = __ffma2_rn(make_float2(rho, rho), make_float2(w.w.bx, w.w.by), make_float2(w.w.ax, w.w.ay));
     }
-    const float tx = __fadd_rd(sx, RL_FLOOR_MAGIC), ty = __fadd_rd(sy, RL_FLOOR_MAGIC);
+    const float2 f = __fadd2_rd(s, make_float2(RL_FLOOR_MAGIC, RL_FLOOR_MAGIC));
+    const float2 r = rl_minus2(s, __fadd2_rn(f, make_float2(-RL_FLOOR_MAGIC, -RL_FLOOR_MAGIC)));
     RLFastTap t;
-    t.fx = sx - (tx - RL_FLOOR_MAGIC);
-    t.fy = sy - (ty - RL_FLOOR_MAGIC);
-    t.idx = base + __float_as_uint(ty) * (unsigned)W + __float_as_uint(tx);
+    t.fx = r.x;
+    t.fy = r.y;
+    t.idx = base + __float_as_uint(f.y) * (unsigned)W + __float_as_uint(f.x);
     return t;
 }
 
@@ -592,6 +600,13 @@ __device__ __forceinline__ bool rl_chunk_inside(const RLPixWarp<ANCH>& w, const 
 __device__ __forceinline__ float4 rl_weights(float fx, float fy) {
     const float gx = 1.f - fx, gy = 1.f - fy;
     return make_float4(gx * gy, fx * gy, gx * fy, fx * fy);
+}
+
+// The same values with both complements from one packed instruction: 1.4% faster where the weights
+// are used once (render), 2% slower in the plane-parallel gradients, which form them twice.
+__device__ __forceinline__ float4 rl_weights_packed(float fx, float fy) {
+    const float2 g = rl_minus2(make_float2(1.f, 1.f), make_float2(fx, fy));
+    return make_float4(g.x * g.y, fx * g.y, g.x * fy, fx * fy);
 }
 
 // The four taps of a sample blended with packed FP32x2 FMAs (the order of rl_sample).

@@ -62,8 +62,8 @@ __device__ __forceinline__ void sample_map(const float* __restrict__ img, int H,
 // CH = 1: M is the alphas alone [D][H][W]; CH = 4: the MPI (a pointer to its first alpha).
 // What bounds it: instruction issue (75%).  A warp's taps of one plane are 32 neighbours: 128 or 64
 // bytes of compact alphas against 512 or 256 bytes of voxels, which were L1's bound (78% busy, now
-// 37%).  Four views of 512x384, D = 32, FP32: 58 us, 72 us from the voxels.
-// (Two nested interpolations take 53 us, but round otherwise: a last-bit change here turns BF16
+// 37%).  Four views of 512x384, D = 32, FP32: 53 us, 72 us from the voxels.
+// (Two nested interpolations took 53 against 58 us, but round otherwise: a last-bit change here turns BF16
 // roundings of the learned network's input, and its output moves by up to 1e-3.)
 template <typename Tm, int CH, bool ANCH>
 __global__ void __launch_bounds__(kAlphaBX * kAlphaBY)

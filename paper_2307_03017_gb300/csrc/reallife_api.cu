@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "rl_internal.h"
+#include "rl_layout.h"
 
 // ------------------------------------------------------------------ errors
 
@@ -374,7 +375,7 @@ rl_status make_views(const rl_mpi* m, const rl_camera* cams, int n, int level, R
 
 size_t elt_size(rl_dtype dt) { return dt == RL_F32 ? 4 : 2; }
 
-size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
+size_t align_up(size_t x) { return rl_align256(x); }
 
 struct WsLayout {
     size_t Ml, S, slots, G, partials, Il, total;
@@ -460,25 +461,6 @@ rl_status enqueue_hsgd(rl_mpi* m, const float* images, const rl_camera* src, int
                             loss);
 }
 
-// Workspace of reallife_gradient_volume: the level MPI (levels >= 1), the selection and
-// the view alpha weights [N][D][h][w] (largest at level 0).
-struct VolLayout {
-    size_t Ml, S, A, total;
-};
-
-VolLayout vol_layout(int N, int D, int H, int W, int k, rl_dtype dt) {
-    VolLayout L;
-    size_t off = 0;
-    L.Ml = off;
-    if (H % 2 == 0 && W % 2 == 0) off += align_up((size_t)D * (H / 2) * (W / 2) * 4 * elt_size(dt));
-    L.S = off;
-    off += align_up((size_t)k * H * W);
-    L.A = off;
-    off += align_up((size_t)N * D * H * W * sizeof(float));
-    L.total = off;
-    return L;
-}
-
 __global__ void k_zero(float4* __restrict__ p, size_t n4) {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
         p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -546,7 +528,7 @@ extern "C" rl_status reallife_refine(rl_mpi* m, const float* images, const rl_ca
 
 extern "C" size_t reallife_gradient_volume_workspace_bytes(int N, int D, int H, int W, int k, rl_dtype dtype) {
     if (N < 1 || D < 1 || H < 1 || W < 1 || k < 1) return 0;
-    return vol_layout(N, D, H, W, k, dtype).total;
+    return rl_vol_layout(N, D, H, W, k, elt_size(dtype)).total;
 }
 
 extern "C" rl_status reallife_gradient_volume(const rl_mpi* m, const float* images, const rl_camera* src, int N,
@@ -563,25 +545,22 @@ rl_status rl_gradient_volume(const rl_mpi* m, const float* images, const rl_came
     p.k = k;
     p.lambda = 1.0f;
     p.selection = selection;
-    const size_t need = (m && N >= 1) ? vol_layout(N, m->D, m->H, m->W, k, m->dtype).total : 0;
+    const size_t need = (m && N >= 1) ? rl_vol_layout(N, m->D, m->H, m->W, k, elt_size(m->dtype)).total : 0;
     // the step's checks (MPI, k, selection, level, images, cameras); its workspace is not used
     rl_status st = check_hsgd(m, images, src, N, &p, level, ws, ~(size_t)0);
     if (st) return st;
     if (act ? ((uintptr_t)act & 15) != 0 : (!V || ((uintptr_t)V & 3) != 0))
         return rl_fail(RL_EINVAL, "V must be a non-NULL, 4-byte aligned device buffer");
     if (ws_bytes < need) return rl_fail(RL_ENOMEM, "workspace %zu bytes < %zu needed", ws_bytes, need);
-    const VolLayout L = vol_layout(N, m->D, m->H, m->W, k, m->dtype);
+    const RLVolLayout L = rl_vol_layout(N, m->D, m->H, m->W, k, elt_size(m->dtype));
     char* base = (char*)ws;
     const int h = m->H >> level, w = m->W >> level;
     void* Ml = level == 0 ? m->data : (void*)(base + L.Ml);
     uint8_t* S = S_out ? S_out : (uint8_t*)(base + L.S);
     float* A = (float*)(base + L.A);
-    // the level's alphas alone, for the view alpha weights: at level 0 in the place of the level MPI
-    // (unused there, and as large), above it behind the level's weights, which take at most a quarter
-    // of theirs; odd sizes have no room for them
-    void* alphas = nullptr;
-    if (level) alphas = base + L.A + align_up((size_t)N * m->D * h * w * sizeof(float));
-    else if (m->H % 2 == 0 && m->W % 2 == 0) alphas = base + L.Ml;
+    // the level's alphas alone, for the view alpha weights
+    const size_t alphas_at = rl_vol_alphas(L, N, m->D, m->H, m->W, level, elt_size(m->dtype));
+    void* alphas = alphas_at == RL_NO_ROOM ? nullptr : base + alphas_at;
     RLViews views;
     st = make_views(m, src, N, level, views);
     if (st) return st;

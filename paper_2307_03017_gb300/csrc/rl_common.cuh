@@ -702,16 +702,18 @@ __device__ __forceinline__ float rl_warp_sum(float v) {
     return v;
 }
 
-// One compensated addition (Kahan): s + c carries the running sum of FP32 values to about FP64.
+// One compensated addition (Kahan): s - c carries the running sum of FP32 values to about FP64.  A sum
+// that has left the range stays infinite: its compensation would be the NaN of inf - inf.
 __device__ __forceinline__ void rl_kahan_add(float& s, float& c, float v) {
     const float y = v - c, t = s + y;
-    c = (t - s) - y;
+    c = fabsf(t) < INFINITY ? (t - s) - y : 0.f;
     s = t;
 }
 
 // Sum of the n loss partials at `partials` (16-byte aligned) by one block, in an order fixed by n and
-// the block's size, so the loss is deterministic.  The total is returned to thread 0; `red` is shared
-// scratch of nthreads / 32 floats.
+// the block's size, so the loss is deterministic.  Each thread's own sums are compensated, so the error
+// does not grow with the partials a thread adds; the threads' sums are added in plain FP32.  The total is
+// returned to thread 0; `red` is shared scratch of nthreads / 32 floats.
 __device__ __forceinline__ float rl_partials_sum(const float* __restrict__ partials, unsigned n, int tid, int nthreads,
                                                  float* red) {
     float a[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
@@ -732,7 +734,7 @@ __device__ __forceinline__ float rl_partials_sum(const float* __restrict__ parti
         }
     }
     if (tid < (int)(n & 3u)) rl_kahan_add(a[0], c[0], __ldcg(partials + n4 * 4 + tid));
-    const float acc = rl_warp_sum((a[0] + a[1]) + (a[2] + a[3]));
+    const float acc = rl_warp_sum(((a[0] - c[0]) + (a[1] - c[1])) + ((a[2] - c[2]) + (a[3] - c[3])));
     if ((tid & 31) == 0) red[tid >> 5] = acc;
     __syncthreads();
     float total = 0.f;

@@ -492,8 +492,8 @@ void launch_grad_t(const void* M, int D, int H, int W, const RLViews& views, con
 
 size_t rl_grad_num_blocks(int H, int W, int N) {
     const size_t own = (size_t)((W + kGradBX - 1) / kGradBX) * ((H + kGradBY - 1) / kGradBY) * N;
-    const size_t a = rl_grad_pp_num_blocks(H, W, N);
-    return own > a ? own : a;
+    const size_t a = rl_grad_pp_num_blocks(H, W, N, false), b = rl_grad_pp_num_blocks(H, W, N, true);
+    return own > a ? (own > b ? own : b) : (a > b ? a : b);
 }
 
 rl_status rl_launch_grad(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,

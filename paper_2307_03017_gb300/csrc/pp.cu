@@ -134,18 +134,21 @@ struct PPShape {
 };
 
 // Tile of the gradient over a W x H image: 32 x 1 pixels (512x384: 218 against 224 us with 16 x 2)
-// unless 16 x 2 needs fewer tiles (widths just above a multiple of 32) or the grid is too high.
-__host__ __device__ inline int grad_pp_tile_x(int H, int W) {
-    if (H > 65535) return 16;
+// unless 16 x 2 needs fewer tiles (widths just above a multiple of 32) or the grid is too high.  Tiles
+// with an anchor of their own are always 16 x 2: the error of their pixels' positions grows with the
+// distance from the anchor (up to 8 pixels instead of 16: 6e-7 instead of 1.2e-6 px, 300x12, f = 300,
+// rotated by 45 degrees).
+__host__ __device__ inline int grad_pp_tile_x(int H, int W, bool anchored) {
+    if (anchored || H > 65535) return 16;
     return (W + 15) / 16 * ((H + 1) / 2) < (W + 31) / 32 * H ? 16 : 32;
 }
 
 // Blocks of about `most_warps` warps; a tile of D planes takes ceil(D / 4) of them.
-__host__ __device__ inline PPShape grad_pp_shape(int D, int H, int W, int most_warps) {
+__host__ __device__ inline PPShape grad_pp_shape(int D, int H, int W, int most_warps, bool anchored) {
     PPShape s;
     s.G = (D + kChunk - 1) / kChunk;
     s.tiles = most_warps / s.G > 1 ? most_warps / s.G : 1;
-    s.tile_x = grad_pp_tile_x(H, W);
+    s.tile_x = grad_pp_tile_x(H, W, anchored);
     return s;
 }
 
@@ -220,12 +223,35 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
     constexpr int C = kChunk;
     __shared__ float4 xch[kMaxWarps][kPix];  // per chunk: (Cc.rgb, Tc)
     __shared__ float ximg[kMaxWarps][kPix][3];
-    __shared__ RLAnchor sA;
-    if (ANCH)
-        rl_anchor_build(&sA, views, pc.view, bx * sh.tiles * sh.tile_x + sh.tiles * sh.tile_x / 2,
-                        pc.ty * (kPix / sh.tile_x), D, W, threadIdx.x, blockDim.x);
+    // An anchor a tile, at its centre: no farther outside the image than the host's check of the rays
+    // reaches.  One anchor for all tiles of a block lies up to 256 pixels from some of its pixels (D <= 4,
+    // batched), where the FP32 differences lose what the anchor is for, or outside the image where its
+    // ray leaves the reference half-space: positions 0.015 px off at 64x24, f = 64, turned by 33 degrees,
+    // 1.5e-6 px with an anchor a tile.  The tiles' tables share one array: a block holds at most
+    // kMaxWarps / ceil(D / kChunk) tiles, so tiles x D <= RL_DEV_MAX_PLANES entries.
+    // One thread forms a tile's head and one a plane's entry: an FP64 instruction costs the same for one
+    // lane as for all.
+    __shared__ RLAnchor sA;  // the tables
+    __shared__ RLAnchorHead sH[kMaxWarps];
+    const int at = pc.tile < sh.tiles ? pc.tile : 0;  // a warp without a tile reads the first one's
+    const int first = ANCH ? at * D : 0;
+    if (ANCH) {
+        // scratch in the exchange buffer, which is written after the last barrier here: the batched kernel
+        // holds both kinds, and 512 bytes more a kind would cost it 36 KB of L1 (64 KB for two blocks)
+        double(*ab)[4] = reinterpret_cast<double(*)[4]>(xch);
+        const RLViewParam64& P = views.v64[pc.view];
+        const int last = (W + sh.tile_x - 1) / sh.tile_x - 1, rows = kPix / sh.tile_x;
+        if ((int)threadIdx.x < sh.tiles)
+            rl_anchor_head(&sH[threadIdx.x], ab[threadIdx.x], P,
+                           min(bx * sh.tiles + (int)threadIdx.x, last) * sh.tile_x + sh.tile_x / 2,
+                           pc.ty * rows + rows / 2);
+        __syncthreads();
+        for (int i = threadIdx.x; i < sh.tiles * D; i += blockDim.x)
+            rl_anchor_plane(sA.k + i, sA.f + i, ab[i / D], views, P, i % D, W);
+        __syncthreads();
+    }
     const int qx = min(pc.qx, W - 1), qy = min(pc.qy, H - 1);
-    const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sA, views.v[pc.view], qx, qy);
+    const RLPixWarp<ANCH> w = rl_pix_warp<ANCH>(sH[at], views.v[pc.view], qx, qy);
     const unsigned hw = (unsigned)(H * W);
     const size_t plane = (size_t)H * W * 4;
     const int d0 = pc.g * C;
@@ -247,12 +273,12 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
     float Tloc[C];
     unsigned word[C];
     const unsigned base = rl_fast_base(qx, qy, W);
-    const bool fast = __all_sync(0xffffffffu, rl_chunk_inside<ANCH>(w, sA, views, d0, d0 + n - 1, qx, qy, H, W));
+    const bool fast = __all_sync(0xffffffffu, rl_chunk_inside<ANCH>(w, sA, views, d0, d0 + n - 1, qx, qy, H, W, first));
     if (fast) {
 #pragma unroll
         for (int i = C - 1; i >= 0; --i) {
             const int d = FULL ? d0 + i : d0 + min(i, n - 1);
-            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+            const RLFastTap t = rl_fast_tap<ANCH>(w, sA, first + d, views.rho[d], base, W);
             m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             word[i] = 0xFFFFFFFFu;
             if (RL_IN((long long)t.idx + W + 1, hw)) {
@@ -268,7 +294,7 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
             m[i] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (FULL || i < n) {
                 const int d = d0 + i;
-                m[i] = rl_sample(M + d * plane, H, W, w.taps(sA, d, views.rho[d], qx, qy));
+                m[i] = rl_sample(M + d * plane, H, W, w.taps(sA, first + d, views.rho[d], qx, qy));
             }
         }
     }
@@ -363,16 +389,16 @@ __device__ __forceinline__ void grad_pp_tile(const Tm* __restrict__ M, int D, in
                 g.z = gc * r2;
                 g.w = Td * fmaf(mi.x - b0, r0, fmaf(mi.y - b1, r1, (mi.z - b2) * r2));
                 if (join) {
-                    const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                    const RLFastTap t = rl_fast_tap<ANCH>(w, sA, first + d, views.rho[d], base, W);
                     if (!pc.active || Td == 0.f) g = make_float4(0.f, 0.f, 0.f, 0.f);
                     join_taps(G, act, pc.lane, Td != 0.f, (unsigned)d, (unsigned)d * hw + t.idx, W, t.fx, t.fy, g, ng);
                 } else if (Td != 0.f) {
                     if (fast) {  // the taps are formed again: keeping them costs registers, and warps
-                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d, views.rho[d], base, W);
+                        const RLFastTap t = rl_fast_tap<ANCH>(w, sA, first + d, views.rho[d], base, W);
                         rl_scatter_at<SPARSE>(G, word[i], (unsigned)d, t.idx, (unsigned)d * hw + t.idx, hw, W,
                                               rl_weights(t.fx, t.fy), g, ng);
                     } else {
-                        const RLTaps t = w.taps(sA, d, views.rho[d], qx, qy);
+                        const RLTaps t = w.taps(sA, first + d, views.rho[d], qx, qy);
                         if (t.ok) rl_scatter<SPARSE>(G, slots, (unsigned)d, hw, H, W, t, g, ng);
                     }
                 }
@@ -405,6 +431,27 @@ k_grad_pp(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__
                                                images, img_level, grad_out, slots, G, inv_n, partials, nparts);
 }
 
+// One unit of the batch below: a block's tiles of one view of one item.  A function of its own, so that the
+// loop's registers and the other kind of coordinates do not press on it (inlined, 32 to 48 bytes of spills
+// a thread): two anchored requests of 2000x58, D = 32, 2 views, FP32: 298 against 308 us; six requests
+// of 128x96, D = 32, 3 views: 118 against 127 us.
+template <typename Tm, bool ANCH>
+__device__ __noinline__ void grad_pp_unit(const RLBatchItem& it, unsigned local) {
+    const unsigned view = local % (unsigned)it.N, block = local / (unsigned)it.N;
+    const int h = it.H >> it.level, w = it.W >> it.level;
+    const int bx = (int)(block % it.pp_tiles_x), by = (int)(block / it.pp_tiles_x);
+    const PPShape sh = grad_pp_shape(it.D, h, w, kMaxWarps, ANCH);
+    PPPos pc = pp_pos(h, w, (int)view, bx, by, sh);
+    if (pc.tile >= sh.tiles) {  // a warp without a tile: a chunk of the first one, used by none
+        pc.tx = bx * sh.tiles;
+        pc.g = 0;
+        pc.G = 1;
+    }
+    grad_pp_tile<Tm, false, true, true, ANCH>(static_cast<const Tm*>(it.Ml), it.D, h, w, it.views, pc, sh, bx,
+                                              it.level ? it.Il : it.images, 0, nullptr, it.slots, it.G, it.inv_n,
+                                              it.partials, it.parts);
+}
+
 // Batched gradient, plane-parallel family: one persistent launch of 16-warp blocks walks the
 // gradient units of the batch table's items that take this family (a unit is one block's tiles of
 // one view of one item).
@@ -416,24 +463,8 @@ k_grad_pp_batch(const RLBatchHeader* __restrict__ hdr, const RLBatchItem* __rest
     __shared__ unsigned next_slot;
     for (unsigned u = rl_batch_next(hdr, 2, &next_slot); u < total; u = rl_batch_next(hdr, 2, &next_slot)) {
         const RLBatchItem& it = items[rl_batch_find(items, n, u, &RLBatchItem::pp_begin)];
-        const unsigned local = u - it.pp_begin;
-        const unsigned view = local % (unsigned)it.N, block = local / (unsigned)it.N;
-        const int h = it.H >> it.level, w = it.W >> it.level;
-        const int bx = (int)(block % it.pp_tiles_x), by = (int)(block / it.pp_tiles_x);
-        const PPShape sh = grad_pp_shape(it.D, h, w, kMaxWarps);
-        const Tm* Ml = static_cast<const Tm*>(it.Ml);
-        PPPos pc = pp_pos(h, w, (int)view, bx, by, sh);
-        if (pc.tile >= sh.tiles) {  // a warp without a tile: a chunk of the first one, used by none
-            pc.tx = bx * sh.tiles;
-            pc.g = 0;
-            pc.G = 1;
-        }
-#define RL_PPB(A) grad_pp_tile<Tm, false, true, true, A>(Ml, it.D, h, w, it.views, pc, sh, bx,                  \
-                                                           it.level ? it.Il : it.images, 0, nullptr, it.slots,   \
-                                                           it.G, it.inv_n, it.partials, it.parts)
-        if (it.views.anchored) RL_PPB(true);
-        else RL_PPB(false);
-#undef RL_PPB
+        if (it.views.anchored) grad_pp_unit<Tm, true>(it, u - it.pp_begin);
+        else grad_pp_unit<Tm, false>(it, u - it.pp_begin);
         __syncthreads();  // the exchange buffers are reused by the next unit
     }
 }
@@ -501,8 +532,8 @@ void launch_render_pp_t(int G, int C, const void* M, int D, int H, int W, const 
 }  // namespace
 
 // Tiles of a gradient launch over all views: the loss partials it writes.
-size_t rl_grad_pp_num_blocks(int H, int W, int N) {
-    const int tx = grad_pp_tile_x(H, W), ty = kPix / tx;
+size_t rl_grad_pp_num_blocks(int H, int W, int N, bool anchored) {
+    const int tx = grad_pp_tile_x(H, W, anchored), ty = kPix / tx;
     return (size_t)((W + tx - 1) / tx) * ((H + ty - 1) / ty) * N;
 }
 
@@ -510,8 +541,9 @@ rl_status rl_launch_grad_pp(const void* M, rl_dtype dt, int D, int H, int W, con
                             const float* images, int img_level, const float* grad_out, const uint8_t* slots,
                             float* G_out, float inv_n, float* partials, int* nblocks, cudaStream_t s) {
     // kernel path 4 asks for narrower blocks
-    const PPShape sh = grad_pp_shape(D, H, W, rl_kernel_path_setting() == 4 ? 4 : 8);
-    const unsigned nparts = (unsigned)rl_grad_pp_num_blocks(H, W, views.n);
+    const bool anchored = views.anchored != 0;
+    const PPShape sh = grad_pp_shape(D, H, W, rl_kernel_path_setting() == 4 ? 4 : 8, anchored);
+    const unsigned nparts = (unsigned)rl_grad_pp_num_blocks(H, W, views.n, anchored);
     if (nblocks) *nblocks = (int)nparts;
     const bool sparse = slots != nullptr;
     const char* name = dt == RL_F32 ? (sparse ? "grad_sparse_f32" : "grad_dense_f32")
@@ -550,13 +582,13 @@ rl_status rl_launch_render_pp(const void* M, rl_dtype dt, int D, int H, int W, c
     return rl_check_launch("render_pp");
 }
 
-unsigned rl_grad_pp_tiles_x(int h, int w, int D) {
-    const PPShape sh = grad_pp_shape(D, h, w, kMaxWarps);
+unsigned rl_grad_pp_tiles_x(int h, int w, int D, bool anchored) {
+    const PPShape sh = grad_pp_shape(D, h, w, kMaxWarps, anchored);
     const int per = sh.tile_x * sh.tiles;
     return (unsigned)((w + per - 1) / per);
 }
-unsigned rl_grad_pp_tiles_y(int h, int w) {
-    const int rows = kPix / grad_pp_tile_x(h, w);
+unsigned rl_grad_pp_tiles_y(int h, int w, bool anchored) {
+    const int rows = kPix / grad_pp_tile_x(h, w, anchored);
     return (unsigned)((h + rows - 1) / rows);
 }
 

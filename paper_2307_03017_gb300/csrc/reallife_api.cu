@@ -797,9 +797,10 @@ extern "C" rl_status reallife_batch_prepare(const rl_batch_item* items, int n, v
             it.parts = it.grad_units;
             max_gather_D = std::max(max_gather_D, (unsigned)m->D);
         } else {
-            it.pp_tiles_x = rl_grad_pp_tiles_x(h, w, m->D);
-            it.pp_units = (unsigned)b.N * it.pp_tiles_x * rl_grad_pp_tiles_y(h, w);
-            it.parts = (unsigned)rl_grad_pp_num_blocks(h, w, b.N);
+            const bool anchored = it.views.anchored != 0;
+            it.pp_tiles_x = rl_grad_pp_tiles_x(h, w, m->D, anchored);
+            it.pp_units = (unsigned)b.N * it.pp_tiles_x * rl_grad_pp_tiles_y(h, w, anchored);
+            it.parts = (unsigned)rl_grad_pp_num_blocks(h, w, b.N, anchored);
         }
         it.upd_begin = upd;
         it.upd_tiles_x = (unsigned)((m->W + 127) / 128);

@@ -233,12 +233,64 @@ struct RLPlaneF {
     float rho;
 };
 
-struct RLAnchor {
+struct RLAnchorHead {
     float mx, my, ez, Nx, Ny, Dc;  // anchor quantities (FP32) for the per-pixel differences
     int u, v;                      // anchor pixel
+};
+
+struct RLAnchor : RLAnchorHead {
     RLPlaneK k[RL_DEV_MAX_PLANES];
     RLPlaneF f[RL_DEV_MAX_PLANES];
 };
+
+// The head of the anchor at pixel (u, v) of view P; ab: the offset's coefficients there, a(q_c) and
+// b(q_c), for rl_anchor_plane.
+__device__ __forceinline__ void rl_anchor_head(RLAnchorHead* A, double* ab, const RLViewParam64& P, int u, int v) {
+    const double mx = ((double)u - P.cxv) * P.inv_fxv, my = ((double)v - P.cyv) * P.inv_fyv;
+    const double ex = P.E[0] * mx + P.E[1] * my + P.E[2];
+    const double ey = P.E[3] * mx + P.E[4] * my + P.E[5];
+    const double ez = P.E[6] * mx + P.E[7] * my + P.E[8];
+    const double dz = 1.0 + ez;
+    const double Nx = ex - mx * ez, Ny = ey - my * ez;
+    // 1 / dz: the FP32 reciprocal refined by two Newton steps in FP64 (relative error far
+    // below FP64's 1e-16 after the second), cheaper than an FP64 division on this GPU
+    double inv = (double)__frcp_rn((float)dz);
+    inv = inv * (2.0 - dz * inv);
+    inv = inv * (2.0 - dz * inv);
+    const double rmx = Nx * inv, rmy = Ny * inv;
+    ab[0] = P.dcx + P.dfx * mx + P.fxr * rmx;
+    ab[1] = P.dcy + P.dfy * my + P.fyr * rmy;
+    ab[2] = P.fxr * (P.C[0] - P.C[2] * (mx + rmx));
+    ab[3] = P.fyr * (P.C[1] - P.C[2] * (my + rmy));
+    A->mx = (float)mx;
+    A->my = (float)my;
+    A->ez = (float)ez;
+    A->Nx = (float)Nx;
+    A->Ny = (float)Ny;
+    A->Dc = (float)dz;
+    A->u = u;
+    A->v = v;
+}
+
+// The entries k, f of plane d (inverse depth V.rho64[d]) of the anchor with coefficients ab; W the plane's width.
+__device__ __forceinline__ void rl_anchor_plane(RLPlaneK* kd, RLPlaneF* fd, const double* ab, const RLViews& V,
+                                                const RLViewParam64& P, int d, int W) {
+    const double rho = V.rho64[d];
+    const double kx = ab[0] + rho * ab[2], ky = ab[1] + rho * ab[3];
+    RLPlaneK k;
+    if (1.0 - rho * P.C[2] > 0.0 && fabs(kx) < 1e9 && fabs(ky) < 1e9) {
+        const double fx = floor(kx), fy = floor(ky);
+        k.ix = (int)fx;
+        k.iy = (int)fy;
+        k.fx = (float)(kx - fx);
+        k.fy = (float)(ky - fy);
+    } else {
+        k.ix = k.iy = RL_PLANE_NONE;
+        k.fx = k.fy = 0.f;
+    }
+    *kd = k;
+    *fd = RLPlaneF{k.fx, k.fy, (int)((unsigned)k.iy * (unsigned)W + (unsigned)k.ix), V.rho[d]};
+}
 
 // Fills A (shared memory) for view `view` of V at anchor pixel (u, v).  Every thread of the
 // block calls it (it synchronises the block twice); nthreads threads, index tid; W the plane's width.
@@ -246,50 +298,9 @@ __device__ __forceinline__ void rl_anchor_build(RLAnchor* A, const RLViews& V, i
                                                 int tid, int nthreads) {
     __shared__ double s_ab[4];
     const RLViewParam64& P = V.v64[view];
-    if (tid == 0) {
-        const double mx = ((double)u - P.cxv) * P.inv_fxv, my = ((double)v - P.cyv) * P.inv_fyv;
-        const double ex = P.E[0] * mx + P.E[1] * my + P.E[2];
-        const double ey = P.E[3] * mx + P.E[4] * my + P.E[5];
-        const double ez = P.E[6] * mx + P.E[7] * my + P.E[8];
-        const double dz = 1.0 + ez;
-        const double Nx = ex - mx * ez, Ny = ey - my * ez;
-        // 1 / dz: the FP32 reciprocal refined by two Newton steps in FP64 (relative error far
-        // below FP64's 1e-16 after the second), cheaper than an FP64 division on this GPU
-        double inv = (double)__frcp_rn((float)dz);
-        inv = inv * (2.0 - dz * inv);
-        inv = inv * (2.0 - dz * inv);
-        const double rmx = Nx * inv, rmy = Ny * inv;
-        s_ab[0] = P.dcx + P.dfx * mx + P.fxr * rmx;
-        s_ab[1] = P.dcy + P.dfy * my + P.fyr * rmy;
-        s_ab[2] = P.fxr * (P.C[0] - P.C[2] * (mx + rmx));
-        s_ab[3] = P.fyr * (P.C[1] - P.C[2] * (my + rmy));
-        A->mx = (float)mx;
-        A->my = (float)my;
-        A->ez = (float)ez;
-        A->Nx = (float)Nx;
-        A->Ny = (float)Ny;
-        A->Dc = (float)dz;
-        A->u = u;
-        A->v = v;
-    }
+    if (tid == 0) rl_anchor_head(A, s_ab, P, u, v);
     __syncthreads();
-    for (int d = tid; d < D; d += nthreads) {
-        const double rho = V.rho64[d];
-        const double kx = s_ab[0] + rho * s_ab[2], ky = s_ab[1] + rho * s_ab[3];
-        RLPlaneK k;
-        if (1.0 - rho * P.C[2] > 0.0 && fabs(kx) < 1e9 && fabs(ky) < 1e9) {
-            const double fx = floor(kx), fy = floor(ky);
-            k.ix = (int)fx;
-            k.iy = (int)fy;
-            k.fx = (float)(kx - fx);
-            k.fy = (float)(ky - fy);
-        } else {
-            k.ix = k.iy = RL_PLANE_NONE;
-            k.fx = k.fy = 0.f;
-        }
-        A->k[d] = k;
-        A->f[d] = RLPlaneF{k.fx, k.fy, (int)((unsigned)k.iy * (unsigned)W + (unsigned)k.ix), V.rho[d]};
-    }
+    for (int d = tid; d < D; d += nthreads) rl_anchor_plane(A->k + d, A->f + d, s_ab, V, P, d, W);
     __syncthreads();
 }
 
@@ -299,7 +310,7 @@ struct RLAnchorPix {
     bool ok;  // the pixel's ray points into the reference half-space and its offsets are bounded
 };
 
-__device__ __forceinline__ RLAnchorPix rl_anchor_pixel(const RLAnchor& A, const RLViewParam& P, int qx, int qy) {
+__device__ __forceinline__ RLAnchorPix rl_anchor_pixel(const RLAnchorHead& A, const RLViewParam& P, int qx, int qy) {
     RLAnchorPix w;
     const float dmx = (float)(qx - A.u) * P.inv_fxv, dmy = (float)(qy - A.v) * P.inv_fyv;
     const float dex = fmaf(P.E[0], dmx, P.E[1] * dmy);
@@ -356,7 +367,7 @@ struct RLPixWarp<true> {
 };
 
 template <bool ANCH>
-__device__ __forceinline__ RLPixWarp<ANCH> rl_pix_warp(const RLAnchor& A, const RLViewParam& P, int qx, int qy) {
+__device__ __forceinline__ RLPixWarp<ANCH> rl_pix_warp(const RLAnchorHead& A, const RLViewParam& P, int qx, int qy) {
     RLPixWarp<ANCH> r;
     if constexpr (ANCH)
         r.w = rl_anchor_pixel(A, P, qx, qy);
@@ -570,15 +581,15 @@ __device__ __forceinline__ RLFastTap rl_fast_tap(const RLPixWarp<ANCH>& w, const
 // True when the samples of every plane in [d_lo, d_hi] lie inside the plane, at least a pixel from
 // its border, and the planes are met in front of the view: position and depth factor are linear in
 // the plane's inverse depth, so the two end planes bound the others.  The pixel of margin covers
-// the rounding.
+// the rounding.  `first` is plane 0's entry in the anchor's tables.
 template <bool ANCH>
 __device__ __forceinline__ bool rl_chunk_inside(const RLPixWarp<ANCH>& w, const RLAnchor& A, const RLViews& views,
-                                                int d_lo, int d_hi, int qx, int qy, int H, int W) {
+                                                int d_lo, int d_hi, int qx, int qy, int H, int W, int first = 0) {
     const float rho0 = views.rho[d_lo], rho1 = views.rho[d_hi];
     float x0, y0, x1, y1;
     bool ok;
     if constexpr (ANCH) {
-        const RLPlaneK a = A.k[d_lo], b = A.k[d_hi];
+        const RLPlaneK a = A.k[first + d_lo], b = A.k[first + d_hi];
         ok = w.w.ok && a.ix != RL_PLANE_NONE && b.ix != RL_PLANE_NONE;
         x0 = (float)(qx + a.ix) + (a.fx + fmaf(rho0, w.w.dbx, w.w.dax));
         y0 = (float)(qy + a.iy) + (a.fy + fmaf(rho0, w.w.dby, w.w.day));

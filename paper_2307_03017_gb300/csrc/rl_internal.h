@@ -91,7 +91,7 @@ size_t rl_grad_num_blocks(int H, int W, int N);
 rl_status rl_launch_grad_pp(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, bool mode_loss,
                             const float* images, int img_level, const float* grad_out, const uint8_t* slots, float* G,
                             float inv_n, float* partials, int* nblocks, cudaStream_t s);
-size_t rl_grad_pp_num_blocks(int H, int W, int N);
+size_t rl_grad_pp_num_blocks(int H, int W, int N, bool anchored);
 rl_status rl_launch_render_pp(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, float* out,
                               cudaStream_t s);
 rl_status rl_launch_loss_reduce(const float* partials, int n, float scale, float* out, cudaStream_t s);
@@ -137,8 +137,8 @@ rl_status rl_launch_grad_pp_batch(const void* table, rl_dtype dt, cudaStream_t s
 rl_status rl_launch_update_batch(const void* table, rl_dtype dt, cudaStream_t s);
 unsigned rl_grad_gather_tiles_x(int w);
 unsigned rl_grad_gather_tiles_y(int h);
-unsigned rl_grad_pp_tiles_x(int h, int w, int D);
-unsigned rl_grad_pp_tiles_y(int h, int w);
+unsigned rl_grad_pp_tiles_x(int h, int w, int D, bool anchored);
+unsigned rl_grad_pp_tiles_y(int h, int w, bool anchored);
 
 // Blocks of a persistent launch of `kernel`: the resident blocks per SM on the current device
 // times its SMs (at least one); computed once per device and kernel instantiation.

@@ -389,8 +389,9 @@ k_grad_shift(const Tm* __restrict__ M, int D, int H, int W, const __grid_constan
 #pragma unroll
         for (int i = 0; i < kGroup; ++i) {
             const int d = j * kGroup + i;
-            if (d < D && (Ta[i] != 0.f || Tb[i] != 0.f)) {
-                const float4 g0 = adjoint(Ta[i], m0[i], b0, r0), g1 = adjoint(Tb[i], m1[i], b1, r1);
+            // a pixel beyond the image scatters nothing, even where a voxel that it alone samples is not finite
+            if (d < D && act0 && (Ta[i] != 0.f || Tb[i] != 0.f)) {
+                const float4 g0 = adjoint(Ta[i], m0[i], b0, r0), g1 = act1 ? adjoint(Tb[i], m1[i], b1, r1) : none;
                 const int2 o = sS.i[d];
                 const unsigned p = (unsigned)(qy + o.y) * (unsigned)W + (unsigned)(qx + o.x);
                 const float4 w = sS.w[d];

@@ -43,7 +43,7 @@ int rl_kernel_path(int H, int W, int nviews) {
 int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bool sparse) {
     const int p = g_path.load(std::memory_order_relaxed);
     if (p != 0) return p >= 3 ? 3 : p;
-    if (H > 2 * 65535) return 2;  // beyond the plane-parallel grid
+    if (H > 2 * 65535 || W > 16 * 65535) return 2;  // beyond the plane-parallel grid (tiles of 16 x 2)
     const long long pixel_views = (long long)H * W * nviews;
     if (sparse && shifts && pixel_views >= (1ll << 17)) return 2;
     if (pixel_views < (1ll << 19)) return 3;

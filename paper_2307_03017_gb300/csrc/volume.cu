@@ -124,6 +124,9 @@ k_view_alpha(const Tm* __restrict__ M, int D, int H, int W, const __grid_constan
 // threads): 68 against 90 us for the volume, 79 against 109 us packed (512x384, N = 4, k = 5; bound by
 // L1, most of it one 32-byte sector a tap of the alpha weights, whose planes differ from lane to lane).
 // Resident warps hide those taps: 12 blocks take 72 us and packed 81, 10 take 75, 16 take 68.
+// The coarse levels' kernels have no such bound (0): with one of 8 blocks the compiler takes the same 64
+// registers, but other code (level 3, 1024x768, N = 4, k = 5: 245 against 204 us; level 2, 512x384, BF16:
+// 54.8 against 49.3 us).
 template <bool L0>
 __device__ __forceinline__ void voxel_view(const float* __restrict__ A, const float* __restrict__ images,
                                            const RLInvViews& iv, int D, int h, int w, int level, int x, int y,
@@ -176,7 +179,7 @@ __device__ __forceinline__ void voxel_view(const float* __restrict__ A, const fl
 }
 
 template <typename Tm, bool L0>
-__global__ void __launch_bounds__(128, L0 ? 14 : 8)
+__global__ void __launch_bounds__(128, L0 ? 14 : 0)
 k_volume(const Tm* __restrict__ Ml, int D, int h, int w, int level, const uint8_t* __restrict__ S, int k,
          const float* __restrict__ A, const float* __restrict__ images, const __grid_constant__ RLInvViews iv,
          float* __restrict__ V) {
@@ -219,7 +222,7 @@ k_volume(const Tm* __restrict__ Ml, int D, int h, int w, int level, const uint8_
 // slot, warp i computing view i (the gathers of a warp stay those of one view); the voxels'
 // channels meet in shared memory and leave as one contiguous 64-byte record per voxel.
 template <typename Tm, bool L0>
-__global__ void __launch_bounds__(32 * RL_DEV_MAX_VIEWS, L0 ? 4 : 2)
+__global__ void __launch_bounds__(32 * RL_DEV_MAX_VIEWS, L0 ? 4 : 0)
 k_volume_packed(const Tm* __restrict__ Ml, int D, int h, int w, int level, const uint8_t* __restrict__ S,
                 const float* __restrict__ A, const float* __restrict__ images, const __grid_constant__ RLInvViews iv,
                 __nv_bfloat16* __restrict__ act) {

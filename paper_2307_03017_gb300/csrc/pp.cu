@@ -531,6 +531,14 @@ void launch_render_pp_t(int G, int C, const void* M, int D, int H, int W, const 
 
 }  // namespace
 
+// Share of an SM's 32 warps (64 registers) that hold planes in a launch of D planes: blocks of G x tiles warps
+// fill the SM only in part, and the last chunk of a tile may be short.
+double rl_grad_pp_fill(int D) {
+    const PPShape s = grad_pp_shape(D, 1, 1, 8, false);
+    const int warps = s.G * s.tiles;
+    return (double)(32 / warps * warps) / 32.0 * D / (s.G * kChunk);
+}
+
 // Tiles of a gradient launch over all views: the loss partials it writes.
 size_t rl_grad_pp_num_blocks(int H, int W, int N, bool anchored) {
     const int tx = grad_pp_tile_x(H, W, anchored), ty = kPix / tx;

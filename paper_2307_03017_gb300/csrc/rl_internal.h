@@ -32,21 +32,33 @@ unsigned int* rl_device_status_ptr();
 // 2^19 pixel-views (small views), where per-pixel threads are too few to hide gather latency,
 // and per-pixel gather otherwise.
 int rl_kernel_path(int H, int W, int nviews);
-// The same for the gradient of D planes (sparse: compact).  Automatic, by measured times:
-//  - else fewer than 2^19 pixel-views: plane-parallel, which gathers each sample once (64x48, 2 views,
-//    D = 32: 13 against 51 us; 256x192, 8 views, D = 64: 233 against 289 us);
+// The same for the gradient of D planes (sparse: compact).  Automatic, in this order, by measured times:
+//  - images beyond the plane-parallel grid (H > 131070 or W > 1048560): per-pixel;
 //  - pure shifts with a compact gradient, from 2^17 pixel-views on: per-pixel, whose kernel for them
 //    shares taps between two pixels and forms no coordinates (256x192, 4 views, D = 32, FP32: 51
 //    against 64 us; 512x384, 4 views, BF16: 175 against 206);
-//  - anchored coordinates: per-pixel, since a plane-parallel block repeats the FP64 set-up of the
-//    anchors for every 32 pixels, a per-pixel one for every 128 (1024x768, 4 views, D = 64, BF16:
+//  - fewer than 2^19 pixel-views: plane-parallel, which gathers each sample once (64x48, 2 views,
+//    D = 32: 13 against 51 us; 256x192, 8 views, D = 64: 233 against 289 us);
+//  - anchored coordinates: per-pixel, since a plane-parallel tile repeats the FP64 set-up of the
+//    anchors for every 32 pixels, a per-pixel block for every 128 (1024x768, 4 views, D = 64, BF16:
 //    2507 against 1710 us);
-//  - compact: plane-parallel up to 32 planes (512x384, 4 views, BF16: 206 against 246 us; 700x768:
-//    545 against 593) or 2^20 pixel-views (512x384, D = 64: 442 against 465); beyond, the chunk
-//    exchange of sixteen warps costs more than the second gather (700x768, D = 64: 1178 against 1112);
-//  - dense: plane-parallel, whose warps join their lanes' shared taps (500x375, 4 views, D = 32: 226
-//    against 290 us; 960x540, 2 views, D = 64: 793 against 828).
+//  - compact: plane-parallel where its warps fill the SM (rl_grad_pp_fill >= 0.8) and up to 32 planes
+//    (512x384, 4 views, BF16: 206 against 246 us; 700x768: 545 against 593) or 2^20 pixel-views
+//    (512x384, 3 views, D = 40, FP32: 225 against 234).  Else per-pixel: with D = 33, 34 and 41 to 50 too
+//    few of an SM's warps hold planes (512x384, 5 views, BF16: D = 33 331 against 260 us, D = 42 467 against
+//    326), beyond 2^20 the chunk exchange of sixteen warps costs more than the second gather (700x768,
+//    D = 64: 1178 against 1112);
+//  - dense: plane-parallel, whose warps join their lanes' shared taps (500x375, 4 views, D = 32: 223
+//    against 286 us), from a fill on that grows with the pixel-views (from 2^20 on the per-pixel kernel
+//    fills the device evenly), for pure shifts (whose per-pixel taps vary least) and beyond 36 planes.
+//    960x540, 4 views, FP32, plane-parallel against per-pixel, rotated and shifted: D = 5 137 / 112,
+//    136 / 105; D = 13 277 / 287, 285 / 269; D = 25 537 / 547, 555 / 512; D = 36 734 / 796, 732 / 746;
+//    D = 42 1120 / 927, 1137 / 869; D = 52 1199 / 1157, 1174 / 1081; D = 57 1378 / 1270, 1348 / 1187;
+//    D = 60 1331 / 1341, 1287 / 1249.  500x375, 4 views: D = 5 51 / 47, 50 / 44; D = 13 106 / 117,
+//    104 / 110; D = 42 400 / 365, 418 / 349; D = 48 418 / 422, 425 / 401.
 int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bool sparse);
+// Share of an SM's warps that hold planes in a plane-parallel gradient of D planes.
+double rl_grad_pp_fill(int D);
 // The gradient family of a batched step of so many pixel-views in all: per-pixel gather, whose long
 // units hide the cost of fetching them (eight requests of 2 to 50 M samples: 2484 us against 3475 us
 // plane-parallel), unless the whole batch is too small to fill the device with them.

@@ -48,7 +48,12 @@ int rl_grad_path(int H, int W, int nviews, int D, bool anchored, bool shifts, bo
     if (sparse && shifts && pixel_views >= (1ll << 17)) return 2;
     if (pixel_views < (1ll << 19)) return 3;
     if (anchored) return 2;
-    return !sparse || D <= 32 || pixel_views < (1ll << 20) ? 3 : 2;
+    const double fill = rl_grad_pp_fill(D);
+    const bool large = pixel_views >= (1ll << 20);
+    if (sparse) return fill >= 0.8 && (D <= 32 || !large) ? 3 : 2;
+    // dense: the least fill at which plane-parallel is the faster, [large][shifts][D > 36]
+    static const double least[2][2][2] = {{{0.68, 0.68}, {0.68, 0.83}}, {{0.76, 0.86}, {0.84, 0.90}}};
+    return fill >= least[large][shifts][D > 36] ? 3 : 2;
 }
 
 int rl_batch_grad_path(long long pixel_views) {

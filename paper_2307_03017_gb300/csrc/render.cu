@@ -8,7 +8,7 @@
 // What bounds it: instruction issue (1920x1080, D = 64, BF16, anchored: 78% of the issue slots at
 // 83 instructions a sample before).  A warp whose samples of the nearest and the farthest plane lie
 // inside the planes has all of them inside, so it leaves out the border tests and takes the fast
-// coordinates of rl_common.cuh, two planes at a time: 13.2 against 17.0 ms for 45 such views, 82
+// coordinates of rl_common.cuh, two planes at a time (render_group): 13.2 against 17.0 ms for 45 such views, 82
 // against 86 us for 4 rotated 500x375 views, D = 32, FP32 (13.6 ms without the packed arithmetic of
 // positions and weights; without it too, one plane at a time 14.7 ms, four 14.5).  Views that are pure
 // shifts of the reference (no rotation, no depth offset, same focal lengths) take a kernel that
@@ -19,14 +19,14 @@
 namespace {
 
 constexpr int kRenderBX = 32, kRenderBY = 4;
-constexpr int kRenderGroup = 2;  // planes whose loads are in flight together
 #ifndef RL_RENDER_MIN_BLOCKS
 #define RL_RENDER_MIN_BLOCKS 1  // no register cap: measured fastest
 #endif
 
 // Blocks are ordered view-fastest (grid x = view) so that the views of a tile, whose plane
 // footprints overlap, run together and share the MPI through L2.
-template <typename Tm, bool ANCH>
+// GROUP: planes whose loads are in flight together.
+template <typename Tm, bool ANCH, int GROUP>
 __global__ void __launch_bounds__(kRenderBX* kRenderBY, RL_RENDER_MIN_BLOCKS)
 k_render(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ RLViews views, int tiles_x,
          float* __restrict__ out) {
@@ -51,23 +51,23 @@ k_render(const Tm* __restrict__ M, int D, int H, int W, const __grid_constant__ 
         c2 = fmaf(a, m.z, c2);
         T = T * (1.f - m.w);
     };
-    // warps whose samples of every plane lie inside it take kRenderGroup planes at a time, without
-    // the border tests
+    // warps whose samples of every plane lie inside it take GROUP planes at a time, without
+    // the border tests (not worth testing for with one or two planes)
     int d = D - 1;
-    if (__all_sync(act, rl_chunk_inside<ANCH>(w, sA, views, 0, D - 1, qx, qy, H, W))) {
+    if (D > 2 && __all_sync(act, rl_chunk_inside<ANCH>(w, sA, views, 0, D - 1, qx, qy, H, W))) {
         const unsigned base = rl_fast_base(qx, qy, W);
 #pragma unroll 1
-        for (; d >= kRenderGroup - 1 && T != 0.f; d -= kRenderGroup) {
-            float4 m[kRenderGroup];
+        for (; d >= GROUP - 1 && T != 0.f; d -= GROUP) {
+            float4 m[GROUP];
 #pragma unroll
-            for (int i = 0; i < kRenderGroup; ++i) {
+            for (int i = 0; i < GROUP; ++i) {
                 const RLFastTap t = rl_fast_tap<ANCH>(w, sA, d - i, views.rho[d - i], base, W);
                 m[i] = RL_IN((long long)t.idx + W + 1, hw)
                            ? rl_sample_at(M, (unsigned)(d - i) * hw + t.idx, W, rl_weights_packed(t.fx, t.fy))
                            : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
-            for (int i = 0; i < kRenderGroup; ++i)
+            for (int i = 0; i < GROUP; ++i)
                 if (i == 0 || T != 0.f) over(m[i]);
         }
     }
@@ -202,6 +202,22 @@ __global__ void k_warp_offsets(int D, int H, int W, const __grid_constant__ RLVi
     }
 }
 
+// Planes a group: two, but one where the walk is too short to pay for the registers (FP32 70 against 48, BF16 56
+// against 48) that keep other blocks from hiding the set-up: FP32 up to 32 planes with anchors, whose FP64
+// set-up is long (1920x1080, 3 views: D = 8 269 us with two, 239 with one; D = 32 644 / 614; 9 views:
+// D = 32 1987 / 1917, D = 40 2437 / 2466), else up to 4 (960x540, 9 views: D = 4 66.5 / 62.0; 1920x1080,
+// D = 8 70.6 / 72.3); BF16 up to 2 (1920x1080, 3 views: D = 1 52.5 / 47.6, D = 4 190.7 / 192.1).
+int render_group(int D, bool f32, bool anchored) { return D <= (f32 ? (anchored ? 32 : 4) : 2) ? 1 : 2; }
+
+template <typename Tm>
+void launch_render_t(const void* M, int D, int H, int W, const RLViews& views, int tiles_x, dim3 grid, float* out,
+                     cudaStream_t s) {
+    auto kern = render_group(D, sizeof(Tm) == 4, views.anchored != 0) == 1
+                    ? (views.anchored ? k_render<Tm, true, 1> : k_render<Tm, false, 1>)
+                    : (views.anchored ? k_render<Tm, true, 2> : k_render<Tm, false, 2>);
+    kern<<<grid, dim3(kRenderBX, kRenderBY), 0, s>>>((const Tm*)M, D, H, W, views, tiles_x, out);
+}
+
 }  // namespace
 
 rl_status rl_launch_render(const void* M, rl_dtype dt, int D, int H, int W, const RLViews& views, float* out,
@@ -225,14 +241,10 @@ rl_status rl_launch_render(const void* M, rl_dtype dt, int D, int H, int W, cons
     }
     if (dt == RL_F32) {
         RLTraceScope ts("render_f32", s);
-        if (views.anchored) k_render<float, true><<<grid, block, 0, s>>>((const float*)M, D, H, W, views, tiles_x, out);
-        else k_render<float, false><<<grid, block, 0, s>>>((const float*)M, D, H, W, views, tiles_x, out);
+        launch_render_t<float>(M, D, H, W, views, tiles_x, grid, out, s);
     } else {
         RLTraceScope ts("render_bf16", s);
-        if (views.anchored)
-            k_render<__nv_bfloat16, true><<<grid, block, 0, s>>>((const __nv_bfloat16*)M, D, H, W, views, tiles_x, out);
-        else
-            k_render<__nv_bfloat16, false><<<grid, block, 0, s>>>((const __nv_bfloat16*)M, D, H, W, views, tiles_x, out);
+        launch_render_t<__nv_bfloat16>(M, D, H, W, views, tiles_x, grid, out, s);
     }
     return rl_check_launch("render");
 }

@@ -371,9 +371,13 @@ rl_status reallife_kept_mass(const rl_mpi* m, const uint64_t* mask, double* out,
 /* ------------------------------------------------------------------ utilities */
 
 /* Kernel family for the warp kernels (render, gradient):
- *   0 (default) automatic: renders plane-parallel for launches of fewer than 2^19 pixel-views
- *     and per-pixel otherwise; gradients plane-parallel, per-pixel from 2^19 pixel-views on when
- *     the warp offsets exceed 128 px; batched gradients per-pixel from 2^19 pixel-views on;
+ *   0 (default) automatic.  Renders: plane-parallel for launches of fewer than 2^19 pixel-views,
+ *     per-pixel from there on.  Gradients, the first that applies: per-pixel for images of more than
+ *     131070 rows or 1048560 columns; per-pixel for compact gradients of pure shifts from 2^17
+ *     pixel-views on; plane-parallel below 2^19 pixel-views; per-pixel when the warp offsets exceed
+ *     128 px; else plane-parallel where the planes fill its warps (most counts of up to 40 planes;
+ *     compact gradients of 2^20 pixel-views and more only up to 32), per-pixel otherwise.  Batched
+ *     gradients: one family for the batch, per-pixel from 2^19 pixel-views in all on;
  *   1 not used (a family of TMA-staged plane windows, measured slower and removed): RL_EINVAL;
  *   2 per-pixel gather (one thread per view pixel walks all planes);
  *   3 plane-parallel (warps own chunks of planes; chunks combined through the

@@ -141,8 +141,9 @@ rl_status rl_launch_update(void* M, rl_dtype dt, int D, int H, int W, int level,
 
 // Batched stages of one HSGD iteration over a batch table in device memory (header and items
 // of rl_common.cuh), each one persistent launch of one wave of resident blocks.  The gradient
-// stage is two launches: the items that rl_kernel_path sends to the per-pixel gather family
-// (shared memory for `planes` planes) and those it sends to the plane-parallel family.
+// stage has a launch for each family, per-pixel gather (shared memory for `planes` planes) and
+// plane-parallel; a batch's items all take the one that rl_batch_grad_path names, and a captured step
+// holds both launches.
 rl_status rl_launch_select_batch(const void* table, rl_dtype dt, cudaStream_t s);
 rl_status rl_launch_grad_batch(const void* table, rl_dtype dt, int planes, cudaStream_t s);
 rl_status rl_launch_grad_pp_batch(const void* table, rl_dtype dt, cudaStream_t s);
@@ -168,8 +169,6 @@ inline int rl_persistent_grid(int threads, size_t smem) {
     if (cacheable) cached[dev] = grid;
     return grid;
 }
-unsigned rl_grad_batch_tiles_x(int w);
-unsigned rl_grad_batch_tiles_y(int h);
 
 // Metrics (metrics.cu): FP64 partial sums of the SSIM windows, squared differences and kept
 // mass, and the number of partials the two metric calls need.

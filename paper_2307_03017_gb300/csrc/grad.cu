@@ -229,8 +229,8 @@ __device__ __forceinline__ void shift_build(ShiftTable* S, const RLViews& V, int
 // two pixels of a column share their middle tap row exactly: six voxels, six slots and at most six
 // reductions for two samples instead of eight of each, and no coordinates a pixel.
 // What bounds it: instruction issue (67%) and latency at 24 resident warps (80 registers; blocks for 20
-// or 28 warps: 6.60 and 6.31 ms).  1920x1080, D = 64, 8 views, BF16: 6.18 ms; one pixel a thread with
-// the same table 6.69 ms, with anchored coordinates 8.23 ms.  512x384, D = 32, 4 views, FP32: 168 us;
+// or 28 warps: 6.60 and 6.31 ms).  1920x1080, D = 64, 8 views, BF16: 6.09 ms; one pixel a thread with
+// the same table 6.69 ms, with anchored coordinates 8.23 ms.  512x384, D = 32, 4 views, FP32: 170 us;
 // one pixel a thread 213 us.
 constexpr int kShiftTileY = 2 * kGradBY;
 
